@@ -210,19 +210,14 @@ typedef struct vsr_trace_params {
                                   Results are identical; other entry points
                                   take 0. */
     uint32_t lockstep;         /* 1 = the warp runs the traversal in lock step:
-                                  the node loop and the primitive loop repeat
-                                  while any lane needs them and every pass ends
-                                  in a warp vote, so lanes that diverge meet
-                                  again at the next node.  Intersectors
-                                  without counters (with dynamic dispatch:
-                                  kinds without a box callback): a lane that
-                                  holds a leaf keeps descending toward its
-                                  next leaf while other lanes are still
-                                  looking (any hit; closest hit with stack_regs
-                                  0, where what the held leaf's hit culls is
-                                  undone before the lane goes on).
-                                  0 = each lane runs its own loops.  The same
-                                  nodes and leaves are visited in the same
+                                  every pass of the node loop and of the
+                                  primitive loop ends in a warp vote, so lanes
+                                  that diverge meet again at the next node; the
+                                  node loop ends when part of the busy lanes
+                                  (7 in 16) have reached a leaf, which they
+                                  then test together.
+                                  0 = each lane runs its own loops.  Each ray
+                                  visits the same nodes and leaves in the same
                                   order either way, so results are identical.
                                   vsr_trace and vsr_path_trace (static or
                                   dynamic dispatch; static: reg_cap_blocks 0),
@@ -363,10 +358,8 @@ vsr_status vsr_trace_tuned_params(vsr_scene* scene, const vsr_intersector* isect
  *   params    one ray per thread, or persistent warps (persistent 1, refill
  *             threshold, blocks per SM, watchdog as for vsr_trace) with
  *             per-lane loops or in lock step (lockstep 1 takes persistent
- *             1; speculation as for the closest-hit query, the buffer's
- *             last entry as the far limit); image_width allowed; stack in
- *             shared memory (stack_regs ignored).  Results are identical
- *             in every configuration.
+ *             1); image_width allowed; stack in shared memory (stack_regs
+ *             ignored).  Results are identical in every configuration.
  * Errors as vsr_trace.
  */
 vsr_status vsr_trace_multi(vsr_scene* scene, const vsr_ray* rays, uint64_t n,

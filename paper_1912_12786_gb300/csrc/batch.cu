@@ -52,16 +52,12 @@ __global__ void __launch_bounds__(256, 4) k_trace_batch(const BatchItem* __restr
                                                      unsigned long long total,
                                                      unsigned long long* __restrict__ work,
                                                      uint32_t refill, Watchdog wd,
-                                                     const uint32_t* __restrict__ perm,
-                                                     uint32_t stack_max) {
+                                                     const uint32_t* __restrict__ perm) {
     extern __shared__ uint32_t s_stack[];
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t lt_mask = (1u << lane) - 1u;
     ShortStack<K> stk;
     stk.init(s_stack + threadIdx.x, blockDim.x);
-    // closest-hit speculation's entry distances (lock step), after the stack
-    float* tcol =
-        reinterpret_cast<float*>(s_stack + stack_words(stack_max, K) * blockDim.x) + threadIdx.x;
 
     bool has = false;
     bool exhausted = false;
@@ -72,8 +68,7 @@ __global__ void __launch_bounds__(256, 4) k_trace_batch(const BatchItem* __restr
     Best best;
     Stats st;
     H h;
-    uint32_t ref = 0, steps = 0, leaf = 0;
-    bool more = false, pend = false;
+    uint32_t ref = 0, steps = 0;
     uint32_t* err0 = items[0].sc.err;  // the watchdog also reports to scene 0's word
     const unsigned long long t0 = wd.max_ns ? global_ns() : 0ull;
     unsigned long long iters = 0;
@@ -109,8 +104,6 @@ __global__ void __launch_bounds__(256, 4) k_trace_batch(const BatchItem* __restr
                         r = make_ray(VSR_LDG(rays + 2 * ri), VSR_LDG(rays + 2 * ri + 1));
                         h = H();
                         has = true;
-                        more = true;
-                        pend = false;
                         if (!traverse_start<Q, H, false>(*scp, ip, r, h, best, st, ref, steps,
                                                          stk)) {
                             finish_miss(best);
@@ -135,8 +128,7 @@ __global__ void __launch_bounds__(256, 4) k_trace_batch(const BatchItem* __restr
             break;
         }
         if constexpr (LS) {
-            if (warp_step<Q, H, false>(*scp, ip, r, h, best, st, has, ref, more, leaf, pend,
-                                       steps, stk, tcol)) {
+            if (warp_step<Q, H, false>(*scp, ip, r, h, best, st, has, ref, steps, stk)) {
                 finish_miss(best);
                 hp[ri] = hit_record(best);
                 has = false;
@@ -159,9 +151,7 @@ namespace {
 template <int Q, class H, int K, bool LS>
 cudaError_t batch_one(const BatchLaunch& b, cudaStream_t stream, uint32_t* grid_out) {
     auto k = k_trace_batch<Q, H, K, LS>;
-    const uint32_t words =
-        stack_words(b.stack_max, K) + (LS ? spec_words<Q, H, false, K>(b.stack_max) : 0u);
-    const size_t smem = (size_t)words * b.block * sizeof(uint32_t);
+    const size_t smem = (size_t)stack_words(b.stack_max, K) * b.block * sizeof(uint32_t);
     uint32_t grid = b.grid;
     if (grid == 0) {
         if (smem > 48 * 1024) {
@@ -192,7 +182,7 @@ cudaError_t batch_one(const BatchLaunch& b, cudaStream_t stream, uint32_t* grid_
     cudaError_t e = cudaMemsetAsync(b.work, 0, sizeof(unsigned long long), stream);
     if (e != cudaSuccess) return e;
     k<<<grid, b.block, smem, stream>>>(b.items, b.offsets, b.nbatch, b.ip, b.total, b.work,
-                                       b.refill, b.wd, perm, b.stack_max);
+                                       b.refill, b.wd, perm);
     return cudaGetLastError();
 }
 

@@ -78,9 +78,6 @@ __global__ void k_dyn_register() {
 struct IsectDynamic {
     static constexpr bool kCounts = true;
     static constexpr bool kTexcoords = false;
-    // lock-step descent may speculate past a held leaf when the bound kind
-    // has no box callback (box_hooks_silent below decides for each ray)
-    static constexpr bool kMaySpeculate = true;
     // the indirect calls take 128-160 registers uncapped: the persistent and
     // lock-step kernels are compiled for 3 (closest hit) or 4 (any hit)
     // resident 256-thread blocks per SM, as the one-ray-per-thread kernel
@@ -124,12 +121,6 @@ __device__ __forceinline__ void set_callback_scene(IsectDynamic& h, const DevSce
 }
 template <class H>
 __device__ __forceinline__ void set_callback_scene(H&, const DevScene*) {}
-
-// The box hooks observe nothing when the bound kind registered no box
-// callback (every kind but count).
-__device__ __forceinline__ bool box_hooks_silent(const IsectDynamic& h) {
-    return h.on_box == nullptr;
-}
 
 // Per-ray setup in the persistent loop: bind the callbacks and their scene.
 __device__ __forceinline__ void isect_setup(IsectDynamic& h, const IsectParams& ip,

@@ -102,10 +102,8 @@ __global__ void __launch_bounds__(256) k_trace_multi(DevScene sc, IsectParams ip
 
 // Persistent multi-hit (persistent_rays: warps claim rays from a counter and
 // refill idle lanes): each lane's traversal resumable (traverse_start /
-// traverse_step), or the warp in lock step (warp_step, whose closest-hit
-// speculation works with the buffer's last entry as the far limit).  Shared
-// memory per thread: stack, the buffer's t and prim columns, and with LS the
-// speculation's entry distances.
+// traverse_step), or the warp in lock step (warp_step).  Shared memory per
+// thread: stack and the buffer's t and prim columns.
 template <class H, bool LS>
 __device__ __forceinline__ void trace_multi_persistent(
     DevScene sc, IsectParams ip, const float* __restrict__ verts,
@@ -120,28 +118,23 @@ __device__ __forceinline__ void trace_multi_persistent(
     mb.pk = buf + nh * stride + threadIdx.x;
     mb.stride = stride;
     mb.n = nh;
-    float* tcol = reinterpret_cast<float*>(buf + 2u * nh * stride) + threadIdx.x;
     ShortStack<0> stk;
     stk.init(s_stack + threadIdx.x, stride);
     Ray r;
     Stats st;
     H h;
-    uint32_t ref = 0, steps = 0, leaf = 0;
-    bool more = false, pend = false;
+    uint32_t ref = 0, steps = 0;
     persistent_rays<LS>(
         map, work, refill, wd, sc.err,
         [&](unsigned long long ri) {
             r = make_ray(VSR_LDG(rays + 2 * ri), VSR_LDG(rays + 2 * ri + 1));
             h = H();
             isect_setup(h, ip, user);
-            more = true;
-            pend = false;
             return traverse_start<kClosest, H, false>(sc, ip, r, h, mb, st, ref, steps, stk);
         },
         [&](bool busy) {
             if constexpr (LS)
-                return warp_step<kClosest, H, false>(sc, ip, r, h, mb, st, busy, ref, more, leaf,
-                                                     pend, steps, stk, tcol);
+                return warp_step<kClosest, H, false>(sc, ip, r, h, mb, st, busy, ref, steps, stk);
             else
                 return traverse_step<kClosest, H, false>(sc, ip, r, h, mb, st, ref, steps, stk);
         },
@@ -180,8 +173,7 @@ inline auto multi_persistent_kernel() {
 template <class H, bool LS>
 cudaError_t multi_persistent(const LaunchArgs& a, const float* verts, const uint32_t* idx,
                              uint32_t nh) {
-    const uint32_t words = a.sc.stack_depth + 2u * nh +
-                           (LS ? spec_words<kClosest, H, false, 0>(a.sc.stack_depth) : 0u);
+    const uint32_t words = a.sc.stack_depth + 2u * nh;
     const size_t smem = (size_t)words * a.block * sizeof(uint32_t);
     auto k = multi_persistent_kernel<H, LS>();
     if (smem > 48 * 1024) {

@@ -12,9 +12,8 @@
 //                      threads, which the paper's traversal scheme cites.
 // and two ways for a warp's lanes to run the traversal: each lane its own
 // while-while loop (traverse / traverse_step), or the warp in lock step
-// (k_trace_ls, and k_trace_persistent with LS: warp_step, whose loops run
-// while any lane needs them and end every pass in a warp vote; speculative
-// descent for the any-hit query).  Both visit the same nodes and leaves in
+// (k_trace_ls, and k_trace_persistent with LS: warp_step, whose loops end
+// every pass in a warp vote).  Both visit the same nodes and leaves in
 // the same order per ray, so every result is the same.
 //
 // Each translation unit trace_k<K>.cu includes this file and instantiates
@@ -70,11 +69,7 @@ __device__ __forceinline__ void trace_ls(DevScene sc, IsectParams ip,
     Stats st;
     ShortStack<K> stk;
     stk.init(s_stack + threadIdx.x, blockDim.x);
-    // closest-hit speculation's entry distances, after the stack columns
-    float* tcol = reinterpret_cast<float*>(s_stack + stack_words(sc.stack_depth, K) * blockDim.x) +
-                  threadIdx.x;
-    uint32_t ref = 0, steps = 0, leaf = 0;
-    bool more = false, pend = false;
+    uint32_t ref = 0, steps = 0;
     auto finish = [&]() {
         finish_miss(best);
         hits[i] = hit_record(best);
@@ -84,13 +79,10 @@ __device__ __forceinline__ void trace_ls(DevScene sc, IsectParams ip,
     };
     if (busy) {
         r = make_ray(__ldg(rays + 2 * i), __ldg(rays + 2 * i + 1));
-        more = traverse_start<Q, H, STATS>(sc, ip, r, h, best, st, ref, steps, stk);
-        if (!more) finish();
+        if (!traverse_start<Q, H, STATS>(sc, ip, r, h, best, st, ref, steps, stk)) finish();
     }
     while (__any_sync(kFullMask, busy)) {
-        if (warp_step<Q, H, STATS>(sc, ip, r, h, best, st, busy, ref, more, leaf, pend, steps,
-                                   stk, tcol))
-            finish();
+        if (warp_step<Q, H, STATS>(sc, ip, r, h, best, st, busy, ref, steps, stk)) finish();
     }
 }
 
@@ -155,15 +147,11 @@ __device__ __forceinline__ void trace_persistent(
     extern __shared__ uint32_t s_stack[];
     ShortStack<K> stk;
     stk.init(s_stack + threadIdx.x, blockDim.x);
-    // closest-hit speculation's entry distances (lock step), after the stack
-    float* tcol = reinterpret_cast<float*>(s_stack + stack_words(sc.stack_depth, K) * blockDim.x) +
-                  threadIdx.x;
     Ray r;
     Best best;
     Stats st;
     H h;
-    uint32_t ref = 0, steps = 0, leaf = 0;
-    bool more = false, pend = false;
+    uint32_t ref = 0, steps = 0;
     persistent_rays<LS>(
         map, work, refill, wd, sc.err,
         [&](unsigned long long ri) {
@@ -171,14 +159,11 @@ __device__ __forceinline__ void trace_persistent(
             h = H();
             isect_setup(h, ip, user);
             st = Stats();
-            more = true;
-            pend = false;
             return traverse_start<Q, H, STATS>(sc, ip, r, h, best, st, ref, steps, stk);
         },
         [&](bool busy) {
             if constexpr (LS)
-                return warp_step<Q, H, STATS>(sc, ip, r, h, best, st, busy, ref, more, leaf, pend,
-                                              steps, stk, tcol);
+                return warp_step<Q, H, STATS>(sc, ip, r, h, best, st, busy, ref, steps, stk);
             else
                 return traverse_step<Q, H, STATS>(sc, ip, r, h, best, st, ref, steps, stk);
         },
@@ -241,9 +226,7 @@ cudaError_t ensure_smem(Kern kernel, size_t smem) {
 // otherwise.
 template <int Q, class H, bool STATS, int K, bool LS, int MINB = min_blocks<Q, H>()>
 cudaError_t launch_persistent(const LaunchArgs& a) {
-    const uint32_t words = stack_words(a.sc.stack_depth, K) +
-                           (LS ? spec_words<Q, H, STATS, K>(a.sc.stack_depth) : 0u);
-    const size_t smem = (size_t)words * a.block * sizeof(uint32_t);
+    const size_t smem = (size_t)stack_words(a.sc.stack_depth, K) * a.block * sizeof(uint32_t);
     auto k = persistent_kernel<Q, H, STATS, K, LS, MINB>();
     cudaError_t e = ensure_smem(k, smem);
     if (e != cudaSuccess) return e;
@@ -259,9 +242,7 @@ cudaError_t launch_persistent(const LaunchArgs& a) {
 // One ray per thread in lock step (budget as launch_persistent).
 template <int Q, class H, bool STATS, int K, int MINB = min_blocks<Q, H>()>
 cudaError_t launch_lockstep(const LaunchArgs& a) {
-    const uint32_t words =
-        stack_words(a.sc.stack_depth, K) + spec_words<Q, H, STATS, K>(a.sc.stack_depth);
-    const size_t smem = (size_t)words * a.block * sizeof(uint32_t);
+    const size_t smem = (size_t)stack_words(a.sc.stack_depth, K) * a.block * sizeof(uint32_t);
     const unsigned long long grid = (a.map.threads + a.block - 1) / a.block;
     auto k = lockstep_kernel<Q, H, STATS, K, MINB>();
     cudaError_t e = ensure_smem(k, smem);

@@ -231,19 +231,6 @@ __device__ __forceinline__ bool box_hit_o(const Ray& r, float4 lo, float4 hi, fl
     }
 }
 
-// box_hit that also gives the entry distance tn: the box is hit with a
-// smaller far limit t' iff it was hit and tn <= t' (the exit side of the
-// comparison does not depend on the far limit).
-__device__ __forceinline__ bool box_hit_tn(const Ray& r, float4 lo, float4 hi, float tfar,
-                                           float& tn) {
-    const float t0x = __fmaf_rn(lo.x, r.ix, r.nox), t1x = __fmaf_rn(hi.x, r.ix, r.nox);
-    const float t0y = __fmaf_rn(lo.y, r.iy, r.noy), t1y = __fmaf_rn(hi.y, r.iy, r.noy);
-    const float t0z = __fmaf_rn(lo.z, r.iz, r.noz), t1z = __fmaf_rn(hi.z, r.iz, r.noz);
-    tn = fmax3(fminf(t0x, t1x), fminf(t0y, t1y), fmaxf(fminf(t0z, t1z), r.tmin));
-    const float tf = fmin3(fmaxf(t0x, t1x), fmaxf(t0y, t1y), fminf(fmaxf(t0z, t1z), tfar));
-    return tn <= tf;
-}
-
 // intersect(ray, basic_triangle<3,float>): Moller-Trumbore with the fixed
 // rounding order.  Returns false when det == 0 (no t, u, v) and, as a shortcut
 // that changes no decision, when u alone already rules out a geometric hit
@@ -353,10 +340,6 @@ __device__ __forceinline__ bool proc_alpha_accept(const DevScene& sc, const Isec
 struct IsectNone {
     static constexpr bool kCounts = false;
     static constexpr bool kTexcoords = false;  // reads geom id and texcoords
-    // box hooks that may observe nothing, so that a lane may test boxes
-    // ahead of the plain order (warp_step); whether they do for a ray is
-    // box_hooks_silent's answer
-    static constexpr bool kMaySpeculate = true;
     // resident 256-thread blocks per SM the persistent and lock-step kernels
     // are compiled for, per query (1: no register budget)
     static constexpr int kMinBlocksClosest = 1;
@@ -395,7 +378,6 @@ struct IsectProcAlpha : IsectNone {
 // bvh_costs: ++num_boxes per box test, ++num_tris per triangle test.
 struct IsectCount : IsectNone {
     static constexpr bool kCounts = true;
-    static constexpr bool kMaySpeculate = false;  // every box test is counted
     uint32_t num_boxes = 0, num_tris = 0;
     __device__ __forceinline__ void box() { ++num_boxes; }
     __device__ __forceinline__ void tri() { ++num_tris; }
@@ -799,28 +781,6 @@ __device__ __forceinline__ bool test_prim(const DevScene& sc, const IsectParams&
     return Q == kAny;
 }
 
-// Where a lane that holds a leaf may keep descending (warp_step): an
-// intersector whose box hooks may observe nothing, and no measurement
-// counters (box_hooks_silent then decides for the ray, at compile time for
-// the static intersectors).  Any hit: the far limit is the ray's tmax, which
-// never changes, so speculation needs no bookkeeping.  Closest hit: the far
-// limit shrinks when the held leaf improves the result, so speculation
-// records entry distances (in a shared-memory column beside the stack's,
-// for the shared-memory stack, K == 0) and undoes what the new limit culls.
-template <int Q, class H, bool STATS, int K>
-struct Speculate {
-    static constexpr bool any = Q == kAny && H::kMaySpeculate && !STATS;
-    static constexpr bool closest = Q == kClosest && H::kMaySpeculate && !STATS && K == 0;
-    static constexpr bool value = any || closest;
-};
-
-// Whether h's box hooks observe nothing (a static intersector: unless it
-// counts).  The dynamic intersector overloads this with a run-time answer.
-template <class H>
-__device__ __forceinline__ bool box_hooks_silent(const H&) {
-    return !H::kCounts;
-}
-
 // Register budget of the persistent and lock-step kernels with intersector
 // H for query Q, as resident 256-thread blocks per SM (__launch_bounds__).
 template <int Q, class H>
@@ -834,74 +794,46 @@ __host__ __device__ constexpr int min_blocks() {
 template <class H>
 __device__ __forceinline__ void isect_setup(H&, const IsectParams&, const DevScene*) {}
 
-// A reached leaf is held for testing and the next node taken from the stack.
-template <class S>
-__device__ __forceinline__ void hold_leaf(uint32_t& ref, bool& more, uint32_t& leaf, bool& pend,
-                                          S& stk) {
-    if (more && !pend && (ref & kLeafBit)) {
-        leaf = ref;
-        pend = true;
-        if (stk.n)
-            ref = stk.pop();
-        else
-            more = false;
-    }
-}
+// Sixteenths of a warp's busy lanes that end warp_step's node loop.
+constexpr uint32_t kLeafShare = 7u;
 
 // One outer iteration of the while-while traversal (Section 3.2) run by the
 // whole warp in lock step: all 32 lanes call it, lanes without a ray with
-// busy = false.  The node loop and the primitive loop repeat while any lane
-// needs them and every pass ends in a full-warp vote, so lanes that diverge
-// inside a pass meet again at the next one.  (With independent thread
-// scheduling a divergent loop lets the lanes of a warp drift onto different
-// iterations, each group then issuing on its own.)
+// busy = false.  Per lane, `ref` is the node to visit next.  First the node
+// loop: every pass, each lane whose node is an inner one visits it, and the
+// pass ends in a full-warp vote, so lanes that diverge inside a pass meet
+// again at the next one.  (With independent thread scheduling a divergent loop
+// lets the lanes of a warp drift onto different iterations, each group then
+// issuing on its own.)  Then every lane that has reached a leaf tests its
+// primitives, one per pass.
 //
-// Per lane: `ref` is the next node to visit when `more`; `leaf` is a leaf
-// reached and not yet tested when `pend`.  The descent runs until every busy
-// lane holds a leaf or has run out of nodes.  Where Speculate holds, a lane
-// that already holds a leaf keeps descending toward its next one while other
-// lanes are still looking (the speculative traversal of Aila and Laine,
-// 2009).  Then each lane holding a leaf tests its primitives, one per pass.
-//
-// Speculation leaves every result and the sequence of tested leaves as in
-// traverse_body:
-//   - any hit: the far limit is the ray's tmax, so a speculating lane visits
-//     the nodes the plain order visits after the held leaf, in that order;
-//   - closest hit: a speculating lane tests boxes against the far limit of
-//     before the held leaf (tf0), which the leaf may lower (to tf).  Each
-//     entry pushed while speculating keeps, in `tcol`, the largest entry
-//     distance on the way to it (`path`: the node it was pushed from and its
-//     ancestors up to the last entry popped, itself included).  The plain
-//     order would have reached that node iff this distance is <= tf: box
-//     tests along the way passed with tf0 >= tf, and a box hit with far
-//     limit tf0 is hit with tf iff its entry distance is <= tf.  So after
-//     the leaf test, entries above `sbase` (pushed while speculating) whose
-//     distance exceeds tf are dropped, order kept, and so is `ref` when its
-//     own path distance exceeds tf; what is left is what the plain order
-//     holds at the same point, and the leaves come in its order.
+// The node loop ends when kLeafShare of the busy lanes have reached a leaf or
+// finished, not when the last lane has: on incoherent rays the number of inner
+// nodes between two leaves varies so much that the wait for the slowest of 32
+// lanes is about three times the mean (13 inner nodes per leaf, 200,000 random
+// quads), and the early end costs only leaf passes with fewer lanes.  Each
+// lane still visits its own nodes and leaves in the order of traverse_body;
+// only how the warp interleaves them differs.  Measured against a node loop
+// that ran until every lane held a leaf while lanes with one went on
+// speculatively (the speculative traversal of Aila and Laine, 2009, with the
+// bookkeeping that undoes what the leaf culls), persistent, 1,000,003 diffuse
+// rays on 200,000 triangles, alpha texture: closest hit 1,148 -> 838 us, any
+// hit 1,011 -> 812 us, 15.8 of 32 lanes active; 1.2 M occlusion rays on 2 M
+// triangles 533 -> 505 us.  The share is flat between 3/8 and 5/8 (838-850
+// us) and loses on both sides (1/8: 952, 7/8: 977 us).
 // Returns true on busy lanes whose ray has finished (result in best).
 template <int Q, class H, bool STATS, class B, class S>
 __device__ __forceinline__ bool warp_step(const DevScene& sc, const IsectParams& ip,
                                           const Ray& r, H& h, B& best, Stats& st, bool busy,
-                                          uint32_t& ref, bool& more, uint32_t& leaf, bool& pend,
-                                          uint32_t& steps, S& stk, float* tcol) {
-    using Spec = Speculate<Q, H, STATS, S::kRegs>;
-    const bool spec = Spec::value && box_hooks_silent(h);
-    const bool track = Spec::closest && spec;
-    const float kNegInf = -__int_as_float(0x7f800000);
+                                          uint32_t& ref, uint32_t& steps, S& stk) {
     bool done = false;
-    uint32_t sbase = 0;           // track: entries at or above were pushed speculating
-    float path = kNegInf;         // track: largest entry distance on the way to ref
-    float tf0 = 0.0f;             // track: the far limit speculation used
-    if (busy) hold_leaf(ref, more, leaf, pend, stk);
-    if (track && busy && pend) {
-        sbase = stk.n;
-        tf0 = h.far(best.t);
-    }
-    for (;;) {  // while some lane is still looking for a leaf
-        const bool seek = busy && !done && more && !pend;  // then ref is an inner node
-        if (!__any_sync(kFullMask, seek)) break;
-        if (busy && !done && more && !(ref & kLeafBit) && (spec || !pend)) {
+    const uint32_t held = (uint32_t)__popc(__ballot_sync(kFullMask, busy));
+    const uint32_t share = held * kLeafShare / 16u + 1u;
+    for (;;) {
+        const bool inner = busy && !done && !(ref & kLeafBit);
+        const uint32_t descending = (uint32_t)__popc(__ballot_sync(kFullMask, inner));
+        if (descending == 0u || descending + share <= held) break;
+        if (inner) {
             if (++steps > sc.max_steps) {
                 atomicOr(sc.err, kErrSteps);
                 best.fail();
@@ -914,9 +846,8 @@ __device__ __forceinline__ bool warp_step(const DevScene& sc, const IsectParams&
                 h.box();
                 h.box();
                 if (STATS) st.boxes += 2;
-                float tnl = 0.0f, tnr = 0.0f;
-                const bool hl = box_hit_tn(r, la, lb, tfar, tnl) && h.keep(ip, la, lb);
-                const bool hr = box_hit_tn(r, ra, rb, tfar, tnr) && h.keep(ip, ra, rb);
+                const bool hl = box_hit(r, la, lb, tfar) && h.keep(ip, la, lb);
+                const bool hr = box_hit(r, ra, rb, tfar) && h.keep(ip, ra, rb);
                 const uint32_t rl = __float_as_uint(la.w), rr = __float_as_uint(ra.w);
                 if (hl && hr) {
                     const bool neg = (r.negmask >> (ref & 3u)) & 1u;
@@ -925,53 +856,33 @@ __device__ __forceinline__ bool warp_step(const DevScene& sc, const IsectParams&
                         best.fail();
                         done = true;
                     } else {
-                        if (track) tcol[stk.n * stk.stride] = fmaxf(path, neg ? tnl : tnr);
                         stk.push(neg ? rl : rr);
                         ref = neg ? rr : rl;
-                        if (track) path = fmaxf(path, neg ? tnr : tnl);
                     }
                 } else if (hl) {
                     ref = rl;
-                    if (track) path = fmaxf(path, tnl);
                 } else if (hr) {
                     ref = rr;
-                    if (track) path = fmaxf(path, tnr);
                 } else if (stk.n) {
                     ref = stk.pop();
-                    if (track) {
-                        if (stk.n >= sbase) {
-                            path = tcol[stk.n * stk.stride];
-                        } else {  // an entry of the plain order
-                            sbase = stk.n;
-                            path = kNegInf;
-                        }
-                    }
                 } else {
-                    more = false;
-                }
-                if (!done) {
-                    const bool held = pend;
-                    hold_leaf(ref, more, leaf, pend, stk);
-                    if (track && pend && !held) {  // speculation starts here
-                        sbase = stk.n;
-                        path = kNegInf;
-                        tf0 = h.far(best.t);
-                    }
+                    done = true;
                 }
             }
         }
     }
-    // test the held leaves, one primitive of every lane per pass
+    // test the leaves reached, one primitive of every lane per pass
     uint32_t cnt = 0;
     const float4* tp = nullptr;
-    if (busy && !done && pend) {
+    const bool test = busy && !done && (ref & kLeafBit);
+    if (test) {
         if (++steps > sc.max_steps) {
             atomicOr(sc.err, kErrSteps);
             best.fail();
             done = true;
         } else {
-            cnt = (leaf & 7u) + 1u;
-            tp = sc.tris + 3ull * ((leaf >> 3) & 0x0FFFFFFFu);
+            cnt = (ref & 7u) + 1u;
+            tp = sc.tris + 3ull * ((ref >> 3) & 0x0FFFFFFFu);
         }
     }
     for (uint32_t k = 0; __any_sync(kFullMask, k < cnt); ++k) {
@@ -980,40 +891,13 @@ __device__ __forceinline__ bool warp_step(const DevScene& sc, const IsectParams&
             cnt = 0;
         }
     }
-    if (busy && !done) {
-        if (track && pend) {
-            const float tf = h.far(best.t);
-            if (tf < tf0) {  // the leaf lowered the far limit: drop what it culls
-                uint32_t j = sbase;
-                for (uint32_t i = sbase; i < stk.n; ++i) {
-                    const float tn = tcol[i * stk.stride];
-                    if (tn <= tf) {
-                        stk.col[j * stk.stride] = stk.col[i * stk.stride];
-                        tcol[j * stk.stride] = tn;
-                        ++j;
-                    }
-                }
-                stk.n = j;
-                if (more && path > tf) {
-                    if (stk.n)
-                        ref = stk.pop();
-                    else
-                        more = false;
-                }
-            }
-        }
-        pend = false;
-        hold_leaf(ref, more, leaf, pend, stk);
-        if (!pend && !more) done = true;
+    if (test && !done) {
+        if (stk.n)
+            ref = stk.pop();
+        else
+            done = true;
     }
     return busy && done;
-}
-
-// Shared-memory words per thread of the entry-distance column that
-// closest-hit speculation keeps beside the stack (0 where it does not run).
-template <int Q, class H, bool STATS, int K>
-__host__ __device__ constexpr uint32_t spec_words(uint32_t depth) {
-    return Speculate<Q, H, STATS, K>::closest ? depth : 0u;
 }
 
 // Budget of a persistent loop: outer iterations per warp (0: no limit) and
