@@ -34,11 +34,13 @@ struct vsr_scene {
     DevScene dev{};
     DevScene* d_user = nullptr;
     uint32_t* d_err = nullptr;  // [0] device error word; [1] refit box state
-    // kept for updates: leaf order, node ids by tree level (deepest first),
-    // host copies of the texture descriptors
+    // kept for updates: leaf order, the parent of each node pair and its count
+    // of refit arrivals, the refit's root box and box state, host copies of the
+    // texture descriptors
     uint32_t* d_order = nullptr;
-    uint32_t* d_levels = nullptr;
-    std::vector<uint32_t> level_offsets;
+    uint32_t* d_parent = nullptr;
+    uint32_t* d_arrived = nullptr;
+    float4* d_state = nullptr;
     std::vector<TexDesc> h_tex;
     // launch configurations chosen by vsr_trace_tune, per (intersector kind,
     // dispatch, query); read by vsr_trace with params == NULL
@@ -286,32 +288,10 @@ void free_bvh(vsr_scene* s) {
     dfree(s->d_nodes);
     dfree(s->d_tris);
     dfree(s->d_order);
-    dfree(s->d_levels);
-    s->level_offsets.clear();
+    dfree(s->d_parent);
+    dfree(s->d_arrived);
+    dfree(s->d_state);
     s->has_bvh = false;
-}
-
-// Node ids grouped by depth, deepest level first (for the bottom-up refit).
-void node_levels(const vsr_bvh_node* nodes, uint32_t num_nodes, uint32_t max_depth,
-                 std::vector<uint32_t>& ids, std::vector<uint32_t>& offsets) {
-    std::vector<std::vector<uint32_t>> by_depth(max_depth + 1);
-    std::vector<std::pair<uint32_t, uint32_t>> st{{0u, 0u}};
-    while (!st.empty()) {
-        auto [id, depth] = st.back();
-        st.pop_back();
-        by_depth[depth].push_back(id);
-        const uint32_t count = nodes[id].count_axis >> 2;
-        if (count == 0 && id < num_nodes) {
-            st.push_back({nodes[id].left_or_first, depth + 1});
-            st.push_back({nodes[id].left_or_first + 1, depth + 1});
-        }
-    }
-    ids.clear();
-    offsets.assign(1, 0u);
-    for (int dpt = (int)max_depth; dpt >= 0; --dpt) {
-        ids.insert(ids.end(), by_depth[dpt].begin(), by_depth[dpt].end());
-        offsets.push_back((uint32_t)ids.size());
-    }
 }
 
 vsr_status validate_isect(const vsr_intersector* is, int32_t query) {
@@ -750,13 +730,14 @@ vsr_status vsr_bvh_load(vsr_scene* s, const void* blob, size_t bytes) {
             free_bvh(s);
             return cuda_fail(e, "triangle layout");
         }
-        std::vector<uint32_t> ids;
-        node_levels(nodes, num_nodes, max_depth, ids, s->level_offsets);
-        if ((e = dmalloc(&s->d_levels, ids.size())) != cudaSuccess ||
-            (e = cudaMemcpy(s->d_levels, ids.data(), 4ull * ids.size(),
-                            cudaMemcpyHostToDevice)) != cudaSuccess) {
+        if ((e = dmalloc(&s->d_parent, num_nodes / 2u)) != cudaSuccess ||
+            (e = dmalloc(&s->d_arrived, num_nodes / 2u)) != cudaSuccess ||
+            (e = dmalloc(&s->d_state, 2)) != cudaSuccess ||
+            (e = launch_parents(s->d_nodes, num_nodes, s->d_parent, s->d_arrived, nullptr)) !=
+                cudaSuccess ||
+            (e = cudaDeviceSynchronize()) != cudaSuccess) {
             free_bvh(s);
-            return cuda_fail(e, "level list upload");
+            return cuda_fail(e, "refit tables");
         }
     }
     s->num_nodes = num_nodes;
@@ -1352,28 +1333,24 @@ extern "C" vsr_status vsr_scene_update(vsr_scene* s, const float* verts, uint32_
             // word 1 of the error allocation: set by the refit if a box comes
             // out non-finite or inverted
             VSR_CUDA(cudaMemsetAsync(s->d_err + 1, 0, sizeof(uint32_t), cs), "box state");
-            k_build_tris<<<(s->dev.nprims + 255) / 256, 256, 0, cs>>>(s->d_verts, s->d_idx,
-                                                                    s->d_order, s->dev.nprims,
-                                                                    s->d_tris);
-            VSR_CUDA(cudaGetLastError(), "triangle layout");
-            VSR_CUDA(launch_refit(s->d_nodes, s->d_levels, s->level_offsets.data(),
-                                  (uint32_t)s->level_offsets.size() - 1u, s->d_verts, s->d_idx,
-                                  s->d_order, s->d_err + 1, cs),
-                     "refit");
+            const RefitArgs a{s->d_nodes,  s->num_nodes, s->d_verts,  s->d_idx,
+                              s->d_order,  s->d_tris,    s->d_parent, s->d_arrived,
+                              s->d_err + 1, s->d_state,  s->d_user};
+            VSR_CUDA(launch_refit(a, cs), "refit");
         }
     }
-    VSR_CUDA(cudaStreamSynchronize(cs), "update");
     if (verts && s->has_bvh && s->dev.nprims) {
         float4 root[2];
-        VSR_CUDA(cudaMemcpy(root, s->d_nodes, sizeof(root), cudaMemcpyDeviceToHost), "root box");
-        s->dev.root_a = make_float4(root[0].x, root[0].y, root[0].z, 0.0f);
+        VSR_CUDA(cudaMemcpyAsync(root, s->d_state, sizeof(root), cudaMemcpyDeviceToHost, cs),
+                 "root box");
+        VSR_CUDA(cudaStreamSynchronize(cs), "update");
+        s->dev.root_a = root[0];
         s->dev.root_b = make_float4(root[1].x, root[1].y, root[1].z, 0.0f);
         uint32_t unordered = 0;
-        VSR_CUDA(cudaMemcpy(&unordered, s->d_err + 1, sizeof(uint32_t), cudaMemcpyDeviceToHost),
-                 "box state");
+        std::memcpy(&unordered, &root[1].w, sizeof(unordered));
         s->dev.boxes_ordered = unordered ? 0u : 1u;
-        VSR_CUDA(cudaMemcpy(s->d_user, &s->dev, sizeof(DevScene), cudaMemcpyHostToDevice),
-                 "scene descriptor upload");
+    } else {
+        VSR_CUDA(cudaStreamSynchronize(cs), "update");
     }
     return VSR_OK;
 }

@@ -14,7 +14,6 @@
 //             of the Moller-Trumbore solve and through the face normal) and
 //             the texel gradients (through the bilinear weights).
 //
-// Also: the BVH refit used after a vertex update.
 // The shading, adjoint and occlusion kernels use alignment-checked loads
 // (see VSR_LDG).
 #define VSR_CHECKED_LOADS 1
@@ -346,55 +345,6 @@ __global__ void __launch_bounds__(256) k_ao_backward(DevScene sc, ShadeDev sh,
                        g[2] * vis * w[c], vec_texels);
 }
 
-// Bottom-up refit of the node boxes after a vertex update: one launch per
-// tree level, deepest first.  Leaves take the bounds of their triangles'
-// vertices (as the builder does); inner nodes the union of their children.
-// Topology and the packed references are unchanged.
-__global__ void k_refit(float4* __restrict__ nodes, const uint32_t* __restrict__ level_nodes,
-                        uint32_t count, const float* __restrict__ verts,
-                        const uint32_t* __restrict__ idx, const uint32_t* __restrict__ order,
-                        uint32_t* __restrict__ unordered) {
-    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= count) return;
-    const uint32_t id = level_nodes[t];
-    const float4 a = nodes[2ull * id];
-    const uint32_t ref = __float_as_uint(a.w);
-    float lo[3] = {__int_as_float(0x7f800000), __int_as_float(0x7f800000),
-                   __int_as_float(0x7f800000)};
-    float hi[3] = {-lo[0], -lo[1], -lo[2]};
-    if (ref & kLeafBit) {
-        const uint32_t first = (ref >> 3) & 0x0FFFFFFFu, cnt = (ref & 7u) + 1u;
-        for (uint32_t s = first; s < first + cnt; ++s) {
-            const uint32_t p = order[s];
-            for (int k = 0; k < 3; ++k) {
-                const float* v = verts + 3ull * idx[3ull * p + k];
-                for (int c = 0; c < 3; ++c) {
-                    lo[c] = fminf(lo[c], v[c]);
-                    hi[c] = fmaxf(hi[c], v[c]);
-                }
-            }
-        }
-    } else {
-        const uint64_t l = 2ull * (ref >> 2);
-        for (uint64_t c = l; c <= l + 1; ++c) {
-            const float4 ca = nodes[2 * c], cb = nodes[2 * c + 1];
-            lo[0] = fminf(lo[0], ca.x);
-            lo[1] = fminf(lo[1], ca.y);
-            lo[2] = fminf(lo[2], ca.z);
-            hi[0] = fmaxf(hi[0], cb.x);
-            hi[1] = fmaxf(hi[1], cb.y);
-            hi[2] = fmaxf(hi[2], cb.z);
-        }
-    }
-    nodes[2ull * id] = make_float4(lo[0], lo[1], lo[2], a.w);
-    nodes[2ull * id + 1] = make_float4(hi[0], hi[1], hi[2], 0.0f);
-    // the octant-specialised box test needs finite boxes with lo <= hi
-    bool ordered = true;
-    for (int c = 0; c < 3; ++c)
-        ordered = ordered && isfinite(lo[c]) && isfinite(hi[c]) && lo[c] <= hi[c];
-    if (!ordered) atomicOr(unordered, 1u);
-}
-
 cudaError_t launch_shade_hits(const DevScene& sc, const ShadeDev& sh, const float* verts,
                               const uint32_t* idx, const float4* rays, const float4* hits,
                               unsigned long long n, float* image, cudaStream_t stream) {
@@ -419,21 +369,6 @@ cudaError_t render_align_error(unsigned* line) {
     if (e != cudaSuccess || *line == 0) return e;
     const unsigned zero = 0;
     return cudaMemcpyToSymbol(g_vsr_align_line, &zero, sizeof(unsigned));
-}
-
-cudaError_t launch_refit(float4* nodes, const uint32_t* level_nodes,
-                         const uint32_t* level_offsets, uint32_t levels, const float* verts,
-                         const uint32_t* idx, const uint32_t* order, uint32_t* unordered,
-                         cudaStream_t stream) {
-    for (uint32_t l = 0; l < levels; ++l) {
-        const uint32_t begin = level_offsets[l], count = level_offsets[l + 1] - begin;
-        if (count == 0) continue;
-        k_refit<<<(count + 255) / 256, 256, 0, stream>>>(nodes, level_nodes + begin, count, verts,
-                                                         idx, order, unordered);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
 }
 
 cudaError_t launch_ao_shade(const DevScene& sc, const AoArgs& ao, unsigned long long n,

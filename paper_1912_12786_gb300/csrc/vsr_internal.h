@@ -250,13 +250,25 @@ cudaError_t launch_ao_shade(const DevScene& sc, const AoArgs& ao, unsigned long 
 cudaError_t launch_ao_backward(const DevScene& sc, const AoArgs& ao, unsigned long long n,
                                cudaStream_t stream);
 
-// Bottom-up refit over node lists grouped by level, deepest first
-// (level_offsets is a host array of levels + 1 entries).  Any box that comes
-// out non-finite or with lo > hi on some axis ORs 1 into *unordered (the
-// caller zeroes it first).
-cudaError_t launch_refit(float4* nodes, const uint32_t* level_nodes,
-                         const uint32_t* level_offsets, uint32_t levels, const float* verts,
-                         const uint32_t* idx, const uint32_t* order, uint32_t* unordered,
-                         cudaStream_t stream);
+// Refit after a vertex update (refit.cu): triangle layout, node boxes, and the
+// descriptor's root box and box state, in one launch.
+struct RefitArgs {
+    float4* nodes;
+    uint32_t num_nodes;
+    const float* verts;
+    const uint32_t* idx;
+    const uint32_t* order;
+    float4* tris;
+    const uint32_t* parent;  // per pair: the node whose children it holds
+    uint32_t* arrived;       // per pair: climbing threads that have arrived
+    uint32_t* unordered;     // set to 1 if a box comes out non-finite or with
+                             // lo > hi on some axis (the caller zeroes it first)
+    float4* state;           // [2]: the root box, and in [1].w *unordered
+    DevScene* user;          // the scene's descriptor in device memory
+};
+// parent and arrived (num_nodes / 2 words each) of a tree.
+cudaError_t launch_parents(const float4* nodes, uint32_t num_nodes, uint32_t* parent,
+                           uint32_t* arrived, cudaStream_t stream);
+cudaError_t launch_refit(const RefitArgs& a, cudaStream_t stream);
 
 }  // namespace vsr
