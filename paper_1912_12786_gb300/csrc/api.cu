@@ -28,6 +28,7 @@ struct vsr_scene {
     TexDesc* d_tex = nullptr;
     uint8_t* d_texels = nullptr;
     float4* d_nodes = nullptr;
+    uint32_t* d_wide = nullptr;  // two-level node records; null: the binary nodes are walked
     float4* d_tris = nullptr;
     uint32_t num_nodes = 0, max_depth = 0;
     bool has_bvh = false;
@@ -286,6 +287,7 @@ __global__ void k_ao_count(const float4* __restrict__ hits, unsigned long long n
 
 void free_bvh(vsr_scene* s) {
     dfree(s->d_nodes);
+    dfree(s->d_wide);
     dfree(s->d_tris);
     dfree(s->d_order);
     dfree(s->d_parent);
@@ -724,6 +726,13 @@ vsr_status vsr_bvh_load(vsr_scene* s, const void* blob, size_t bytes) {
             k_build_tris<<<(num_prims + 255) / 256, 256>>>(s->d_verts, s->d_idx, s->d_order,
                                                             num_prims, s->d_tris);
             e = cudaGetLastError();
+            // without the memory for the records the binary nodes are walked
+            if (e == cudaSuccess && wide_fits(num_nodes)) {
+                if (dmalloc(&s->d_wide, 8ull * num_nodes) == cudaSuccess)
+                    e = launch_wide_tables(s->d_nodes, num_nodes, s->d_tris, s->d_wide, nullptr);
+                else
+                    cudaGetLastError();
+            }
             if (e == cudaSuccess) e = cudaDeviceSynchronize();
         }
         if (e != cudaSuccess) {
@@ -755,6 +764,7 @@ vsr_status vsr_bvh_load(vsr_scene* s, const void* blob, size_t bytes) {
     d.root_ref = node_ref(nodes[0]);
     d.stack_depth = max_depth > 0 ? max_depth : 1u;
     d.max_steps = num_nodes + 2u;
+    d.wide = s->d_wide;
     d.boxes_ordered = 1u;  // the validator checked every box: finite, lo <= hi
     d.root_a = make_float4(nodes[0].lo[0], nodes[0].lo[1], nodes[0].lo[2], 0.0f);
     d.root_b = make_float4(nodes[0].hi[0], nodes[0].hi[1], nodes[0].hi[2], 0.0f);
@@ -1335,8 +1345,11 @@ extern "C" vsr_status vsr_scene_update(vsr_scene* s, const float* verts, uint32_
             VSR_CUDA(cudaMemsetAsync(s->d_err + 1, 0, sizeof(uint32_t), cs), "box state");
             const RefitArgs a{s->d_nodes,  s->num_nodes, s->d_verts,  s->d_idx,
                               s->d_order,  s->d_tris,    s->d_parent, s->d_arrived,
-                              s->d_err + 1, s->d_state,  s->d_user};
+                              s->d_err + 1, s->d_state,  s->d_user,   s->d_wide};
             VSR_CUDA(launch_refit(a, cs), "refit");
+            if (s->d_wide)
+                VSR_CUDA(launch_build_wide(s->d_nodes, s->num_nodes, s->d_wide, cs),
+                         "node records");
         }
     }
     if (verts && s->has_bvh && s->dev.nprims) {
@@ -1490,6 +1503,7 @@ struct vsr_batch {
     int kind = 0, query = 0;
     IsectParams ip{};
     uint32_t stack_max = 1;
+    bool records = true;  // every scene has two-level node records
     BatchItem* d_items = nullptr;
     unsigned long long* d_offsets = nullptr;
     unsigned long long* d_work = nullptr;
@@ -1604,6 +1618,7 @@ BatchLaunch batch_launch_args(const vsr_batch* b, const vsr_trace_params& p) {
     L.tile_scene = b->d_tile_scene;
     L.sort_ntiles = (uint32_t)b->sort_tiles.size();
     L.lockstep = p.lockstep;
+    L.records = b->records;
     return L;
 }
 
@@ -1791,6 +1806,7 @@ extern "C" vsr_status vsr_batch_create(vsr_scene* const* scenes, const vsr_ray* 
     b->query = query;
     b->ip = isect_params(is);
     b->stack_max = stack_max;
+    for (const BatchItem& it : items) b->records = b->records && it.sc.wide;
     b->shape = shape;
     b->params = prm;
     b->tuned = params != nullptr || tune_lookup(shape, &b->params);

@@ -16,7 +16,7 @@
 // [offsets[s], offsets[s+1]) because the sort key is scene-major.  Per-ray
 // results are identical to a per-scene vsr_trace: the traversal code is the
 // same (traverse_start / traverse_step).
-#include "vsr_internal.h"
+#include "wide.cuh"
 
 namespace vsr {
 
@@ -42,10 +42,14 @@ __device__ __forceinline__ uint32_t scene_of_warp(const unsigned long long* __re
     return lo;
 }
 
+// How a warp runs the traversal: per-lane loops, in lock step over the binary
+// nodes, or in lock step over the two-level records (wide.cuh).
+enum class Walk { kLanes, kLockstep, kRecords };
+
 // Control flow as k_trace_persistent (trace_static.cuh): converged votes at
 // the top of every iteration, one divergent traversal step closed by
 // __syncwarp, uniform exits, and the watchdog.
-template <int Q, class H, int K, bool LS>
+template <int Q, class H, int K, Walk W>
 __global__ void __launch_bounds__(256, 4) k_trace_batch(const BatchItem* __restrict__ items,
                                                      const unsigned long long* __restrict__ offsets,
                                                      uint32_t nbatch, IsectParams ip,
@@ -53,16 +57,18 @@ __global__ void __launch_bounds__(256, 4) k_trace_batch(const BatchItem* __restr
                                                      unsigned long long* __restrict__ work,
                                                      uint32_t refill, Watchdog wd,
                                                      const uint32_t* __restrict__ perm) {
-    extern __shared__ uint32_t s_stack[];
+    constexpr bool kRec = W == Walk::kRecords;
+    extern __shared__ float4 s_mem[];
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t lt_mask = (1u << lane) - 1u;
     ShortStack<K> stk;
-    stk.init(s_stack + threadIdx.x, blockDim.x);
+    stk.init(reinterpret_cast<uint32_t*>(s_mem) + threadIdx.x, blockDim.x);
+    const LaneStore m(s_mem);
+    WideLane<Q, H> w;
 
     bool has = false;
     bool exhausted = false;
-    unsigned long long ri = 0;
-    float4* hp = nullptr;
+    float4* hp = nullptr;  // the lane's hit record
     const DevScene* scp = &items[0].sc;
     Ray r;
     Best best;
@@ -70,8 +76,19 @@ __global__ void __launch_bounds__(256, 4) k_trace_batch(const BatchItem* __restr
     H h;
     uint32_t ref = 0, steps = 0;
     uint32_t* err0 = items[0].sc.err;  // the watchdog also reports to scene 0's word
-    const unsigned long long t0 = wd.max_ns ? global_ns() : 0ull;
-    unsigned long long iters = 0;
+    __shared__ unsigned long long s_t0[kMaxWarps];
+    if (lane == 0) s_t0[threadIdx.x >> 5] = wd.max_ns ? global_ns() : 0ull;
+    __syncwarp();
+    uint32_t iters = 0;
+    auto finish = [&]() {
+        if constexpr (kRec) {
+            *hp = m.hit();
+        } else {
+            finish_miss(best);
+            *hp = hit_record(best);
+        }
+        has = false;
+    };
 
     for (;;) {
         const uint32_t busy = __ballot_sync(kFullMask, has);
@@ -92,7 +109,7 @@ __global__ void __launch_bounds__(256, 4) k_trace_batch(const BatchItem* __restr
                     const unsigned long long g = perm ? (unsigned long long)VSR_LDG(perm + slot)
                                                       : slot;
                     const unsigned long long lo_s = VSR_LDG(offsets + s);
-                    ri = g - lo_s;
+                    const unsigned long long ri = g - lo_s;
                     scp = &items[s].sc;
                     if (perm && (g < lo_s || g >= VSR_LDG(offsets + s + 1))) {
                         // a sorted slot naming a ray of another scene cannot
@@ -100,47 +117,42 @@ __global__ void __launch_bounds__(256, 4) k_trace_batch(const BatchItem* __restr
                         atomicOr(scp->err, kErrHit);
                     } else {
                         const float4* rays = items[s].rays;
-                        hp = items[s].hits;
-                        r = make_ray(VSR_LDG(rays + 2 * ri), VSR_LDG(rays + 2 * ri + 1));
-                        h = H();
-                        has = true;
-                        if (!traverse_start<Q, H, false>(*scp, ip, r, h, best, st, ref, steps,
-                                                         stk)) {
-                            finish_miss(best);
-                            hp[ri] = hit_record(best);
-                            has = false;
+                        hp = items[s].hits + ri;
+                        const float4 a = VSR_LDG(rays + 2 * ri), b = VSR_LDG(rays + 2 * ri + 1);
+                        if constexpr (kRec) {
+                            has = w.start(*scp, ip, a, b, m);
+                        } else {
+                            r = make_ray(a, b);
+                            h = H();
+                            has = traverse_start<Q, H, false>(*scp, ip, r, h, best, st, ref,
+                                                              steps, stk);
                         }
+                        if (!has) finish();
                     }
                 }
             }
         }
         const uint32_t live = __ballot_sync(kFullMask, has);
         if (live == 0u && exhausted) break;
-        if (watchdog_expired(wd, ++iters, t0)) {
+        if (watchdog_expired(wd, ++iters, s_t0 + (threadIdx.x >> 5))) {
             if (lane == 0) atomicOr(err0, kErrTimeout);
             if (has) {
                 atomicOr(scp->err, kErrTimeout);
-                best.fail();
-                finish_miss(best);
-                hp[ri] = hit_record(best);
-                has = false;
+                if constexpr (kRec)
+                    w.fail(m);
+                else
+                    best.fail();
+                finish();
             }
             break;
         }
-        if constexpr (LS) {
-            if (warp_step<Q, H, false>(*scp, ip, r, h, best, st, has, ref, steps, stk)) {
-                finish_miss(best);
-                hp[ri] = hit_record(best);
-                has = false;
-            }
+        if constexpr (kRec) {
+            if (wide_step(*scp, ip, w, m, has)) finish();
+        } else if constexpr (W == Walk::kLockstep) {
+            if (warp_step<Q, H, false>(*scp, ip, r, h, best, st, has, ref, steps, stk)) finish();
         } else {
-            if (has) {
-                if (traverse_step<Q, H, false>(*scp, ip, r, h, best, st, ref, steps, stk)) {
-                    finish_miss(best);
-                    hp[ri] = hit_record(best);
-                    has = false;
-                }
-            }
+            if (has && traverse_step<Q, H, false>(*scp, ip, r, h, best, st, ref, steps, stk))
+                finish();
             __syncwarp();
         }
     }
@@ -148,10 +160,12 @@ __global__ void __launch_bounds__(256, 4) k_trace_batch(const BatchItem* __restr
 
 namespace {
 
-template <int Q, class H, int K, bool LS>
+template <int Q, class H, int K, Walk W>
 cudaError_t batch_one(const BatchLaunch& b, cudaStream_t stream, uint32_t* grid_out) {
-    auto k = k_trace_batch<Q, H, K, LS>;
-    const size_t smem = (size_t)stack_words(b.stack_max, K) * b.block * sizeof(uint32_t);
+    auto k = k_trace_batch<Q, H, K, W>;
+    const size_t smem = W == Walk::kRecords
+                            ? wide_smem(b.block, b.stack_max)
+                            : (size_t)stack_words(b.stack_max, K) * b.block * sizeof(uint32_t);
     uint32_t grid = b.grid;
     if (grid == 0) {
         if (smem > 48 * 1024) {
@@ -186,20 +200,23 @@ cudaError_t batch_one(const BatchLaunch& b, cudaStream_t stream, uint32_t* grid_
     return cudaGetLastError();
 }
 
-template <int Q, class H, bool LS>
+template <int Q, class H, Walk W>
 cudaError_t batch_depth(const BatchLaunch& b, cudaStream_t stream, uint32_t* grid) {
     switch (b.stack_regs) {
-        case 0: return batch_one<Q, H, 0, LS>(b, stream, grid);
-        case 2: return batch_one<Q, H, 2, LS>(b, stream, grid);
-        case 4: return batch_one<Q, H, 4, LS>(b, stream, grid);
+        case 0: return batch_one<Q, H, 0, W>(b, stream, grid);
+        case 2: return batch_one<Q, H, 2, W>(b, stream, grid);
+        case 4: return batch_one<Q, H, 4, W>(b, stream, grid);
         default: return cudaErrorInvalidValue;
     }
 }
 
 template <int Q, class H>
 cudaError_t batch_regs(const BatchLaunch& b, cudaStream_t stream, uint32_t* grid) {
-    return b.lockstep ? batch_depth<Q, H, true>(b, stream, grid)
-                      : batch_depth<Q, H, false>(b, stream, grid);
+    if constexpr (H::kWide)
+        if (b.lockstep && b.stack_regs == 0 && b.records)
+            return batch_one<Q, H, 0, Walk::kRecords>(b, stream, grid);
+    return b.lockstep ? batch_depth<Q, H, Walk::kLockstep>(b, stream, grid)
+                      : batch_depth<Q, H, Walk::kLanes>(b, stream, grid);
 }
 
 template <int Q>

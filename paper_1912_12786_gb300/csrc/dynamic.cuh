@@ -77,6 +77,7 @@ __global__ void k_dyn_register() {
 
 struct IsectDynamic {
     static constexpr bool kCounts = true;
+    static constexpr bool kWide = false;  // the callbacks see every box test
     static constexpr bool kTexcoords = false;
     // the indirect calls take 128-160 registers uncapped: the persistent and
     // lock-step kernels are compiled for 3 (closest hit) or 4 (any hit)

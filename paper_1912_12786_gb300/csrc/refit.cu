@@ -9,7 +9,7 @@
 // That form spent its time on launches (20 levels for 65,000 triangles, 3 to 8
 // us each, most of them with one block); the climb costs a fence and an atomic
 // per level, about 0.7 us.
-#include "vsr_internal.h"
+#include "wide_build.cuh"
 
 namespace vsr {
 
@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(256) k_refit(RefitArgs a) {
         float4* t = a.tris + 3ull * s;
         t[0] = make_float4(v[0][0], v[0][1], v[0][2], __uint_as_float(p));
         t[1] = make_float4(__fsub_rn(v[1][0], v[0][0]), __fsub_rn(v[1][1], v[0][1]),
-                           __fsub_rn(v[1][2], v[0][2]), 0.0f);
+                           __fsub_rn(v[1][2], v[0][2]), __uint_as_float(id));
         t[2] = make_float4(__fsub_rn(v[2][0], v[0][0]), __fsub_rn(v[2][1], v[0][1]),
                            __fsub_rn(v[2][2], v[0][2]), 0.0f);
     }
@@ -94,6 +94,8 @@ __global__ void __launch_bounds__(256) k_refit(RefitArgs a) {
     const uint32_t bad = atomicOr(a.unordered, 0u);
     const float4 ra = make_float4(lo[0], lo[1], lo[2], 0.0f),
                  rb = make_float4(hi[0], hi[1], hi[2], __uint_as_float(bad));
+    if (a.wide)
+        write_wide_header(a.nodes, make_float4(lo[0], lo[1], lo[2], w), rb, !bad, a.wide);
     a.state[0] = ra;
     a.state[1] = rb;
     a.user->root_a = ra;

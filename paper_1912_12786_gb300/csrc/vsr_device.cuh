@@ -7,8 +7,9 @@
 //          inner node are one 64-byte aligned pair (4 x 128-bit loads).
 //   ref    packed node reference: inner = (left/2) << 2 | split axis,
 //          leaf = 1 << 31 | first << 3 | (count - 1).
-//   tris   3 x float4 per leaf slot: {v0.xyz, prim id}, {e1.xyz, 0},
-//          {e2.xyz, 0} with e1 = v1 - v0, e2 = v2 - v0, in leaf order.
+//   tris   3 x float4 per leaf slot: {v0.xyz, prim id}, {e1.xyz, node id of
+//          the leaf}, {e2.xyz, 0} with e1 = v1 - v0, e2 = v2 - v0, in leaf
+//          order.
 //   uvs    3 x float2 per original triangle id; geom: texture id per id.
 //
 // Rounding: the file is compiled with -fmad=false and every product, sum and
@@ -82,7 +83,8 @@ struct DevScene {
     uint32_t max_steps;     // node visits per ray never exceed the node count
     uint32_t boxes_ordered; // 1: every node box is finite with lo <= hi (a
                             // validated blob; rechecked by each refit)
-    uint32_t pad[2];
+    const uint32_t* wide;   // two-level node records (wide.cuh), or null where
+                            // the binary nodes have to be walked
     float4 root_a, root_b;  // root box (lo, hi) in .xyz
 };
 
@@ -340,6 +342,9 @@ __device__ __forceinline__ bool proc_alpha_accept(const DevScene& sc, const Isec
 struct IsectNone {
     static constexpr bool kCounts = false;
     static constexpr bool kTexcoords = false;  // reads geom id and texcoords
+    // no box hooks, and a verdict that depends on the candidate alone: the
+    // two-level node records may be walked (wide.cuh)
+    static constexpr bool kWide = true;
     // resident 256-thread blocks per SM the persistent and lock-step kernels
     // are compiled for, per query (1: no register budget)
     static constexpr int kMinBlocksClosest = 1;
@@ -378,6 +383,7 @@ struct IsectProcAlpha : IsectNone {
 // bvh_costs: ++num_boxes per box test, ++num_tris per triangle test.
 struct IsectCount : IsectNone {
     static constexpr bool kCounts = true;
+    static constexpr bool kWide = false;  // every box test is counted
     uint32_t num_boxes = 0, num_tris = 0;
     __device__ __forceinline__ void box() { ++num_boxes; }
     __device__ __forceinline__ void tri() { ++num_tris; }
@@ -389,6 +395,7 @@ struct IsectCount : IsectNone {
 // the clip box, and a candidate is accepted iff its hit point fmaf(t, d, o)
 // lies in the closed box.
 struct IsectClip : IsectNone {
+    static constexpr bool kWide = false;  // intercepts every box test
     float ox, oy, oz, dx, dy, dz, t_exit;
     __device__ __forceinline__ void begin(const Ray& r, const IsectParams& ip) {
         ox = r.ox;
@@ -904,6 +911,7 @@ __device__ __forceinline__ bool warp_step(const DevScene& sc, const IsectParams&
 // nanoseconds of the global timer per warp (0: no limit).  When either runs
 // out the warp records kErrTimeout, marks its rays in flight as failed and
 // leaves the loop.
+constexpr uint32_t kMaxWarps = 8;  // per block (256 threads)
 struct Watchdog {
     unsigned long long max_iters;
     unsigned long long max_ns;
@@ -917,11 +925,11 @@ __device__ __forceinline__ unsigned long long global_ns() {
 
 // Whether a persistent warp has used up its budget.  Called by all 32 lanes
 // with the same `iters`; the result is the same on every lane.
-__device__ __forceinline__ bool watchdog_expired(const Watchdog& wd, unsigned long long iters,
-                                                 unsigned long long t0) {
+__device__ __forceinline__ bool watchdog_expired(const Watchdog& wd, uint32_t iters,
+                                                 const unsigned long long* t0) {
     if (wd.max_iters && iters > wd.max_iters) return true;
-    if (wd.max_ns && (iters & 255ull) == 0ull)
-        return __any_sync(kFullMask, global_ns() - t0 > wd.max_ns) != 0;
+    if (wd.max_ns && (iters & 255u) == 0u)
+        return __any_sync(kFullMask, global_ns() - *t0 > wd.max_ns) != 0;
     return false;
 }
 
@@ -956,8 +964,12 @@ __device__ __forceinline__ void persistent_rays(const RayMap& map, unsigned long
     bool has = false;        // lane holds a ray in flight
     bool exhausted = false;  // warp-uniform: the counter passed the last slot
     unsigned long long ri = 0;
-    const unsigned long long t0 = wd.max_ns ? global_ns() : 0ull;
-    unsigned long long iters = 0;
+    // the warp's start time and its iterations (32 bits: the limit is one, and
+    // the time is looked at every 256 of them); the time waits in shared memory
+    __shared__ unsigned long long s_t0[kMaxWarps];
+    if (lane == 0) s_t0[threadIdx.x >> 5] = wd.max_ns ? global_ns() : 0ull;
+    __syncwarp();
+    uint32_t iters = 0;
     for (;;) {
         const uint32_t busy = __ballot_sync(kFullMask, has);
         if (!exhausted && (uint32_t)__popc(busy) < refill) {
@@ -978,7 +990,7 @@ __device__ __forceinline__ void persistent_rays(const RayMap& map, unsigned long
         }
         const uint32_t live = __ballot_sync(kFullMask, has);
         if (live == 0u && exhausted) break;
-        if (watchdog_expired(wd, ++iters, t0)) {
+        if (watchdog_expired(wd, ++iters, s_t0 + (threadIdx.x >> 5))) {
             if (lane == 0) atomicOr(err, kErrTimeout);
             if (has) {
                 fail();

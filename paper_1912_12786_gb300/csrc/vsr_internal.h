@@ -49,6 +49,18 @@ struct ShadeDev {
 // register-stack depth).
 cudaError_t launch_static(const LaunchArgs& a, int kind, bool stats);
 cudaError_t launch_static_octant(const LaunchArgs& a, int kind);
+// Two-level node records (wide.cu): whether a tree of num_nodes nodes gets
+// them (64 bytes per node pair); the launches that fill them from the binary
+// nodes -- at load with the header and the triangles' leaf ids, and after a
+// refit, which writes those itself.
+bool wide_fits(uint32_t num_nodes);
+cudaError_t launch_wide_tables(const float4* nodes, uint32_t num_nodes, float4* tris,
+                               uint32_t* wide, cudaStream_t stream);
+cudaError_t launch_build_wide(const float4* nodes, uint32_t num_nodes, uint32_t* wide,
+                              cudaStream_t stream);
+// The static lock-step launches that walk the records (trace_wide.cu).
+bool walks_records(const LaunchArgs& a, int kind);
+cudaError_t launch_wide(const LaunchArgs& a, int kind);
 // Register-stack depths the static kernels are instantiated for.
 bool stack_regs_supported(uint32_t k);
 // The static one-ray-per-thread kernel under __launch_bounds__(256, 3..6)
@@ -202,6 +214,7 @@ struct BatchLaunch {
     const uint32_t* tile_scene = nullptr;  // device [sort_ntiles]: scene of each tile
     uint32_t sort_ntiles = 0;
     uint32_t lockstep = 0;             // 1: the warp runs the traversal in lock step
+    bool records = false;              // every scene has two-level node records
 };
 
 // Coherence order (sort.cu).  coherence_sort_tiles cuts a batch's rays into
@@ -265,6 +278,7 @@ struct RefitArgs {
                              // lo > hi on some axis (the caller zeroes it first)
     float4* state;           // [2]: the root box, and in [1].w *unordered
     DevScene* user;          // the scene's descriptor in device memory
+    uint32_t* wide;          // the two-level records' header, or null
 };
 // parent and arrived (num_nodes / 2 words each) of a tree.
 cudaError_t launch_parents(const float4* nodes, uint32_t num_nodes, uint32_t* parent,
