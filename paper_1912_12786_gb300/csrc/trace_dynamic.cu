@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(256, MINB)
                 const float4* __restrict__ rays, RayMap map, float4* __restrict__ hits,
                 uint2* __restrict__ counters) {
     extern __shared__ uint32_t s_stack[];
-    const unsigned long long g = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned long long g = slot_of_thread(map);
     if (g >= map.threads) return;
     const unsigned long long i = ray_of_thread(g, map);
     if (i >= map.n) return;
@@ -72,7 +72,8 @@ cudaError_t launch_dynamic(const LaunchArgs& a, int kind) {
         return a.query == kClosest ? launch_dynamic_shape<kClosest>(a)
                                    : launch_dynamic_shape<kAny>(a);
     const size_t smem = (size_t)a.sc.stack_depth * a.block * sizeof(uint32_t);
-    const unsigned long long grid = (a.map.threads + a.block - 1) / a.block;
+    RayMap map = a.map;
+    const unsigned long long grid = (spread_rays(map, kSpreadWarpsLarge) + a.block - 1) / a.block;
     const uint32_t cap = a.reg_cap ? a.reg_cap : (a.query == kClosest ? 3u : 4u);
     void (*k)(DevScene, IsectParams, const DevScene*, const float4*, RayMap, float4*, uint2*);
     if (cap == 1)
@@ -88,7 +89,7 @@ cudaError_t launch_dynamic(const LaunchArgs& a, int kind) {
             cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    k<<<(unsigned)grid, a.block, smem, a.stream>>>(a.sc, a.ip, a.dyn_user, a.rays, a.map, a.hits,
+    k<<<(unsigned)grid, a.block, smem, a.stream>>>(a.sc, a.ip, a.dyn_user, a.rays, map, a.hits,
                                                      a.counters);
     return cudaGetLastError();
 }

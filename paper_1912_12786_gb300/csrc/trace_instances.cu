@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(256) k_trace_inst(InstDev is, IsectParams ip,
                                                     uint32_t* __restrict__ inst_ids,
                                                     uint2* __restrict__ counters) {
     extern __shared__ uint32_t s_stack[];
-    const unsigned long long g = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned long long g = slot_of_thread(map);
     if (g >= map.threads) return;
     const unsigned long long i = ray_of_thread(g, map);
     if (i >= map.n) return;
@@ -394,8 +394,9 @@ cudaError_t inst_one(const InstLaunch& L) {
             cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    const unsigned long long grid = (L.map.threads + L.block - 1) / L.block;
-    k<<<(unsigned)grid, L.block, smem, L.stream>>>(L.is, L.ip, L.rays, L.map, L.hits, L.inst_ids,
+    RayMap map = L.map;
+    const unsigned long long grid = (spread_rays(map, kSpreadWarpsLarge) + L.block - 1) / L.block;
+    k<<<(unsigned)grid, L.block, smem, L.stream>>>(L.is, L.ip, L.rays, map, L.hits, L.inst_ids,
                                                    L.counters);
     return cudaGetLastError();
 }

@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(256) k_trace_multi(DevScene sc, IsectParams ip
                                                      uint2* __restrict__ counters,
                                                      const DevScene* __restrict__ user) {
     extern __shared__ uint32_t s_stack[];
-    const unsigned long long g = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned long long g = slot_of_thread(map);
     if (g >= map.threads) return;
     const unsigned long long i = ray_of_thread(g, map);
     if (i >= map.n) return;
@@ -202,8 +202,9 @@ cudaError_t multi_one(const LaunchArgs& a, const float* verts, const uint32_t* i
             cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    const unsigned long long grid = (a.map.threads + a.block - 1) / a.block;
-    k<<<(unsigned)grid, a.block, smem, a.stream>>>(a.sc, a.ip, verts, idx, a.rays, a.map, nh,
+    RayMap map = a.map;
+    const unsigned long long grid = (spread_rays(map, kSpreadWarps) + a.block - 1) / a.block;
+    k<<<(unsigned)grid, a.block, smem, a.stream>>>(a.sc, a.ip, verts, idx, a.rays, map, nh,
                                                      a.hits, a.counters, a.dyn_user);
     return cudaGetLastError();
 }

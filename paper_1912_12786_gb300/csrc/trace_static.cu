@@ -3,6 +3,8 @@
 // each depth K are instantiated in trace_k<K>.cu.
 #include "vsr_internal.h"
 
+#include <atomic>
+
 namespace vsr {
 
 cudaError_t launch_static_k0(const LaunchArgs& a, int kind, bool stats);
@@ -19,7 +21,10 @@ cudaError_t launch_static(const LaunchArgs& a, int kind, bool stats) {
     if (stats) return launch_static_k0(a, kind, true);
     if (a.reg_cap >= 3) return launch_static_capped(a, kind, a.reg_cap);
     if (walks_records(a, kind)) return launch_wide(a, kind);
-    if (a.octant) return launch_static_octant(a, kind);
+    // the octant-dispatching kernel also runs the launches that do not ask for
+    // it (trace_oct.cu)
+    if (a.octant || (!a.persistent && !a.lockstep && a.stack_regs == 0))
+        return launch_static_octant(a, kind);
     switch (a.stack_regs) {
         case 0: return launch_static_k0(a, kind, false);
         case 1: return launch_static_k1(a, kind, false);
@@ -30,10 +35,22 @@ cudaError_t launch_static(const LaunchArgs& a, int kind, bool stats) {
     }
 }
 
-int persistent_grid(uint32_t block, uint32_t blocks_per_sm, const void* kernel, size_t smem) {
-    int dev = 0, sms = 0, per_sm = 0;
+int sm_count() {
+    constexpr int kDevices = 64;
+    static std::atomic<int> known[kDevices];
+    int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (dev >= 0 && dev < kDevices && (sms = known[dev].load(std::memory_order_relaxed)) > 0)
+        return sms;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    if (dev >= 0 && dev < kDevices) known[dev].store(sms, std::memory_order_relaxed);
+    return sms;
+}
+
+int persistent_grid(uint32_t block, uint32_t blocks_per_sm, const void* kernel, size_t smem) {
+    int per_sm = 0;
+    const int sms = sm_count();
+    if (sms <= 0) return 0;
     if (blocks_per_sm) {
         per_sm = (int)blocks_per_sm;
     } else if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, (int)block, smem) !=

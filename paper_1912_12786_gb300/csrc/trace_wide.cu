@@ -11,7 +11,7 @@ __global__ void __launch_bounds__(256, 4) k_trace_wide(DevScene sc, IsectParams 
                                                     const float4* __restrict__ rays, RayMap map,
                                                     float4* __restrict__ hits) {
     extern __shared__ float4 s_lane[];
-    const unsigned long long g = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned long long g = slot_of_thread(map);
     const unsigned long long i = g < map.threads ? ray_of_thread(g, map) : map.n;
     const LaneStore m(s_lane);
     WideLane<Q, H> w;
@@ -59,8 +59,9 @@ cudaError_t wide_one(const LaunchArgs& a) {
         auto k = k_trace_wide<Q, H>;
         cudaError_t e = allow_smem(k, smem);
         if (e != cudaSuccess) return e;
-        const unsigned long long grid = (a.map.threads + a.block - 1) / a.block;
-        k<<<(unsigned)grid, a.block, smem, a.stream>>>(a.sc, a.ip, a.rays, a.map, a.hits);
+        RayMap map = a.map;
+        const unsigned long long grid = (spread_rays(map, kSpreadWarpsLarge) + a.block - 1) / a.block;
+        k<<<(unsigned)grid, a.block, smem, a.stream>>>(a.sc, a.ip, a.rays, map, a.hits);
         return cudaGetLastError();
     }
     auto k = k_trace_wide_persistent<Q, H>;

@@ -102,7 +102,18 @@ struct RayMap {
     unsigned long long threads;  // threads the grid covers
     uint32_t width, tiles_x;
     const uint32_t* perm;        // coherence order, or null
+    uint32_t lane_bits = 5;      // one-ray-per-thread launches: a warp takes
+                                 // 2^lane_bits slots (spread_rays, vsr_internal.h)
 };
+
+// Slot of this thread in a one-ray-per-thread launch, or map.threads when it
+// takes none.
+__device__ __forceinline__ unsigned long long slot_of_thread(const RayMap& m) {
+    const unsigned long long g = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t lane = (uint32_t)g & 31u;
+    const unsigned long long s = ((g >> 5) << m.lane_bits) + lane;
+    return (lane >> m.lane_bits) == 0u && s < m.threads ? s : m.threads;
+}
 
 // Ray of thread g (< map.threads), or map.n when the thread takes none.
 __device__ __forceinline__ unsigned long long ray_of_thread(unsigned long long g,

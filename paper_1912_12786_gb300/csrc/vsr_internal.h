@@ -76,6 +76,31 @@ inline int persistent_grid(const LaunchArgs& a, const void* kernel, size_t smem)
     return persistent_grid(a.block, a.blocks_per_sm, kernel, smem);
 }
 
+// Few rays: fewer of them per warp.  A warp runs the union of its rays' paths
+// and a small launch lasts as long as its slowest warp, so while the chip has
+// room for more warps -- up to warps_per_sm on every SM -- the rays are spread
+// over them.  Measured one ray per thread, closest hit, alpha texture, us at
+// 32 / 16 / 8 / 4 / 2 / 1 rays per warp:
+//   rays     random quads (200,000 triangles)   forest (200,002)
+//   1,000    167 / 135 / 118 / 95 / 76 / 60     77 / 70 / 63 / 62 / 54 / 52
+//   8,000    193 / 156 / 129 / 99 / 77 / 70     80 / 72 / 66 / 62 / 60 / 70
+//   20,000   203 / 154 / 127 / 98 / 88 / 79     99 / 89 / 72 / 76 / 92 / 122
+//   40,960   180 / 150 / 123 / 117 / 112        77 / 76 / 76 / 105 / 142
+//   70,400   172 / 149 / 155 / 141 / 157        74 / 76 / 101 / 145 / 219
+//   100,000  203 / 191 / 154 / 165              81 / 94 / 119 / 184
+// Random quads would take more warps, but neighbouring camera rays that agree
+// (the forest) lose once the warps no longer fit the chip at once: the line is
+// what stays resident, 36 warps of the octant kernels' 56 registers, 24 of the
+// kernels with 78 to 80.  Sets map.lane_bits; returns the launch's threads.
+constexpr unsigned kSpreadWarps = 36, kSpreadWarpsLarge = 24;
+int sm_count();  // of the current device
+inline unsigned long long spread_rays(RayMap& map, unsigned warps_per_sm) {
+    const unsigned long long warps = (unsigned long long)warps_per_sm * (unsigned)sm_count();
+    map.lane_bits = 5;
+    while (map.lane_bits > 0 && (map.threads >> (map.lane_bits - 1)) <= warps) --map.lane_bits;
+    return ((map.threads + (1ull << map.lane_bits) - 1) >> map.lane_bits) * 32ull;
+}
+
 // Run `launch(counter)` with a persistent launch's ray counter, zeroed on
 // `stream` first: `given` when not null, else 8 bytes of stream-ordered
 // scratch freed on the stream after the launch, so persistent launches on
