@@ -213,9 +213,9 @@ typedef struct vsr_trace_params {
                                   every pass of the node loop and of the
                                   primitive loop ends in a warp vote, so lanes
                                   that diverge meet again at the next node; the
-                                  node loop ends when part of the busy lanes
-                                  (7 in 16) have reached a leaf, which they
-                                  then test together.
+                                  node loop ends when the lanes that reached a
+                                  leaf have waited long enough, and they test
+                                  their leaves together.
                                   0 = each lane runs its own loops.  Each ray
                                   visits the same nodes and leaves in the same
                                   order either way, so results are identical.
@@ -391,12 +391,11 @@ vsr_status vsr_trace_multi(vsr_scene* scene, const vsr_ray* rays, uint64_t n,
  *             segments to pixel tiles; persistent launches, lock step and
  *             the octant box test apply to each segment depth; ray_order 0
  * One closest-hit launch per segment depth plus one shading launch, on
- * `stream`.  After each bounce but the last, three small launches compact
- * the live paths (n < 2^32): the next segment's threads take the live paths
- * first, in index order, and the finished ones (inactive rays, dropped at
- * the root box test) after them; results do not depend on it.  Scratch
- * (n * 64 bytes plus 4 bytes per 256 paths) comes from the stream-ordered
- * allocator.  Errors as vsr_trace.
+ * `stream`.  The shading launch also lists the paths that go on (their order
+ * may vary from run to run; results do not depend on it), and the next
+ * segment's threads take the paths of that list.  Scratch (n * 68 bytes; 16
+ * without bounces) comes from the stream-ordered allocator.  Errors as
+ * vsr_trace.
  */
 typedef struct vsr_path_params {
     uint32_t bounces;      /* 0..64 */
@@ -751,7 +750,8 @@ const char* vsr_last_error(void);
 /* Read and clear the scene's device error word (synchronous).
  *   bit 0: a traversal stack overflowed;
  *   bit 1: a ray made more visits than the BVH has nodes (persistent and
- *          batched launches count every node, the others count leaves);
+ *          batched launches with per-lane loops count every node, the others
+ *          count leaves);
  *   bit 2: a render or backward kernel found a load whose address did not
  *          match its width and skipped it (vsr_last_error() names the line);
  *   bit 3: a caller-supplied hit record named a primitive out of range

@@ -273,18 +273,6 @@ __global__ void k_ao_rays(const float* __restrict__ verts, const uint32_t* __res
     }
 }
 
-// Occluded rays per pixel from the ambient-occlusion rays' any-hit records
-// (pixel i's rays at i * spp .. i * spp + spp - 1), as integers, so the
-// counts do not depend on the traversal order.
-__global__ void k_ao_count(const float4* __restrict__ hits, unsigned long long n, uint32_t spp,
-                           uint32_t* __restrict__ cnt) {
-    const unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    uint32_t c = 0;
-    for (uint32_t k = 0; k < spp; ++k) c += __float_as_uint(hits[i * spp + k].w) != kMiss;
-    cnt[i] = c;
-}
-
 void free_bvh(vsr_scene* s) {
     dfree(s->d_nodes);
     dfree(s->d_wide);
@@ -1235,20 +1223,19 @@ extern "C" vsr_status vsr_render_ao(vsr_scene* s, const vsr_ray* rays, uint64_t 
     cudaError_t e = launch_static(a, is->kind, false);
     if (e != cudaSuccess) return cuda_fail(e, "ao primary trace launch");
     // occlusion: the AO rays (as vsr_make_ao_rays makes them) and their
-    // any-hit records in stream-ordered scratch, traced by the trace kernels
-    // at the configuration tuned for this scene, intersector and the any-hit
-    // query (else the default), then counted per pixel
+    // any-hit records in stream-ordered scratch (with a ray counter), traced by
+    // the trace kernels at the configuration tuned for this scene, intersector
+    // and the any-hit query, else the default
     const uint64_t m = n * spp;
-    float4* ao_rays = nullptr;
-    float4* ao_hits = nullptr;
-    e = cudaMallocAsync(reinterpret_cast<void**>(&ao_rays), m * 32, a.stream);
-    if (e == cudaSuccess) e = cudaMallocAsync(reinterpret_cast<void**>(&ao_hits), m * 16, a.stream);
-    if (e == cudaSuccess) {
-        k_ao_rays<<<(unsigned)((n + 255) / 256), 256, 0, a.stream>>>(
-            s->d_verts, s->d_idx, a.rays, ao.hits, n, spp, ao.xi, ao_tmax, eps, s->dev.nprims,
-            s->dev.err, ao_rays);
-        e = cudaGetLastError();
-    }
+    uint8_t* scratch = nullptr;
+    e = cudaMallocAsync(reinterpret_cast<void**>(&scratch), m * 48 + 16, a.stream);
+    if (e != cudaSuccess) return cuda_fail(e, "ao occlusion");
+    float4* ao_rays = reinterpret_cast<float4*>(scratch);
+    float4* ao_hits = ao_rays + 2 * m;
+    k_ao_rays<<<(unsigned)((n + 255) / 256), 256, 0, a.stream>>>(
+        s->d_verts, s->d_idx, a.rays, ao.hits, n, spp, ao.xi, ao_tmax, eps, s->dev.nprims,
+        s->dev.err, ao_rays);
+    e = cudaGetLastError();
     if (e == cudaSuccess) {
         LaunchArgs b = a;
         b.query = VSR_ANY;
@@ -1256,22 +1243,19 @@ extern "C" vsr_status vsr_render_ao(vsr_scene* s, const vsr_ray* rays, uint64_t 
         b.n = m;
         b.hits = ao_hits;
         b.counters = nullptr;
+        b.work = reinterpret_cast<unsigned long long*>(ao_hits + m);
         vsr_trace_params tp;
-        if (!tuned_params(s, is, VSR_ANY, &tp) || tp.image_width) tp = kDefaultParams;
+        const bool tuned = tuned_params(s, is, VSR_ANY, &tp) && !tp.image_width;
+        if (!tuned) tp = kDefaultParams;
         if (apply_params(b, m, tp) != VSR_OK) e = cudaErrorInvalidValue;
         if (e == cudaSuccess)
             e = tp.ray_order ? launch_ordered(b, is->kind, false) : launch_static(b, is->kind, false);
     }
-    if (e == cudaSuccess) {
-        k_ao_count<<<(unsigned)((n + 255) / 256), 256, 0, a.stream>>>(
-            ao_hits, n, spp, reinterpret_cast<uint32_t*>(occlusion));
-        e = cudaGetLastError();
-    }
-    if (ao_hits) cudaFreeAsync(ao_hits, a.stream);
-    if (ao_rays) cudaFreeAsync(ao_rays, a.stream);
+    ao.ao_hits = ao_hits;
+    if (e == cudaSuccess) e = launch_ao_shade(a.sc, ao, n, a.stream);
+    const cudaError_t fr = cudaFreeAsync(scratch, a.stream);
+    if (e == cudaSuccess) e = fr;
     if (e != cudaSuccess) return cuda_fail(e, "ao occlusion");
-    e = launch_ao_shade(a.sc, ao, n, a.stream);
-    if (e != cudaSuccess) return cuda_fail(e, "ao shade launch");
     return VSR_OK;
 }
 
@@ -2190,43 +2174,49 @@ extern "C" vsr_status vsr_path_trace(vsr_scene* s, const vsr_ray* rays, uint64_t
     cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
     DeviceGuard g(s->device);
     if (!g.ok) return fail(VSR_ERR_CUDA, "cannot select the scene's device");
-    float4* work = nullptr;
-    float4* hits = nullptr;
-    float* f = nullptr;
-    // after each bounce the live paths are compacted to the front of a
-    // permutation the next segment's trace follows (ray indices are 32-bit)
-    const bool compact = pp->bounces > 0 && n <= 0xFFFFFFFFull;
-    uint32_t* perm = nullptr;
-    uint32_t* counts = nullptr;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&work), n * 32, cs);
-    if (e == cudaSuccess) e = cudaMallocAsync(reinterpret_cast<void**>(&hits), n * 16, cs);
-    if (e == cudaSuccess) e = cudaMallocAsync(reinterpret_cast<void**>(&f), n * 12, cs);
-    if (e == cudaSuccess && compact)
-        e = cudaMallocAsync(reinterpret_cast<void**>(&perm), n * 4, cs);
-    if (e == cudaSuccess && compact)
-        e = cudaMallocAsync(reinterpret_cast<void**>(&counts),
-                            (path_compact_blocks(n) + 1ull) * 4, cs);
-    if (e == cudaSuccess)
-        e = launch_path_init(reinterpret_cast<const float4*>(rays), n, work, f, radiance, segments,
-                             cs);
-    a.rays = work;
-    a.hits = hits;
+    // path indices are 32-bit; more paths than that would not fit the device
+    if (pp->bounces && n > 0xFFFFFFFFull) return fail(VSR_ERR_OOM, "path scratch allocation");
+    // one allocation: next segments, hits, throughputs, two lists, live counts,
+    // ray counter
+    const uint64_t m = pp->bounces ? n : 0;
+    const uint64_t at_hits = 32 * m, at_f = at_hits + 16 * n, at_list = at_f + 12 * m,
+                   at_live = (at_list + 8 * m + 15) & ~15ull, at_work = at_live + 4 * 64,
+                   bytes = at_work + 8;
+    uint8_t* scratch = nullptr;
+    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&scratch), bytes, cs);
+    if (e == cudaSuccess) e = cudaMemsetAsync(scratch + at_live, 0, 4 * 64, cs);
+    PathBuffers b{};
+    b.verts = s->d_verts;
+    b.idx = s->d_idx;
+    b.rays = reinterpret_cast<const float4*>(rays);
+    b.dirs = dirs;
+    b.radiance = radiance;
+    b.segments = segments;
+    b.work = reinterpret_cast<float4*>(scratch);
+    b.hits = reinterpret_cast<float4*>(scratch + at_hits);
+    b.f = reinterpret_cast<float*>(scratch + at_f);
+    b.list[0] = reinterpret_cast<uint32_t*>(scratch + at_list);
+    b.list[1] = b.list[0] + m;
+    b.live = reinterpret_cast<uint32_t*>(scratch + at_live);
+    a.rays = b.rays;
+    a.hits = b.hits;
     a.stream = cs;
+    a.work = reinterpret_cast<unsigned long long*>(scratch + at_work);
     for (uint32_t k = 0; e == cudaSuccess && k <= pp->bounces; ++k) {
-        if (k == 1 && compact) a.map = RayMap{n, n, 0u, 0u, perm};
+        if (k == 1) {
+            a.rays = b.work;
+        }
+        if (k > 0) {
+            a.map = RayMap{n, n, 0u, 0u, b.list[(k - 1) & 1]};
+        }
         e = is->dispatch == VSR_DISPATCH_STATIC ? launch_static(a, is->kind, false)
                                                 : launch_dynamic(a, is->kind);
-        if (e == cudaSuccess)
-            e = launch_path_bounce(s->dev, pd, s->d_verts, s->d_idx, work, hits, f, dirs, k, n,
-                                   radiance, segments, cs);
-        if (e == cudaSuccess && compact && k < pp->bounces)
-            e = launch_path_compact(f, n, counts, perm, cs);
+        // list entries past the live paths name no ray
+        if (e == cudaSuccess && k < pp->bounces)
+            e = cudaMemsetAsync(b.list[k & 1], 0xFF, 4 * n, cs);
+        if (e == cudaSuccess) e = launch_path_bounce(s->dev, pd, b, k, n, cs);
     }
-    if (counts) cudaFreeAsync(counts, cs);
-    if (perm) cudaFreeAsync(perm, cs);
-    if (f) cudaFreeAsync(f, cs);
-    if (hits) cudaFreeAsync(hits, cs);
-    if (work) cudaFreeAsync(work, cs);
+    if (scratch) cudaFreeAsync(scratch, cs);
     if (e != cudaSuccess)
         return e == cudaErrorMemoryAllocation ? fail(VSR_ERR_OOM, "path scratch allocation")
                                               : cuda_fail(e, "path tracing launch");

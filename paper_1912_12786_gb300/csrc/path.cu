@@ -1,10 +1,10 @@
 // Diffuse path tracing on the closest-hit query with the custom intersector
 // (a workload of many incoherent segments; the paper has no shading).  The
 // host runs it wavefront-style: for each bounce, one closest-hit launch over
-// every path (the trace kernels; finished paths carry an inactive ray that
-// leaves at the root box test), then k_path_bounce, which shades the hits and
-// writes the next segment in place.  FP32 with the operation order fixed, so
-// every bounce reproduces the oracle's bit for bit:
+// the live paths (the trace kernels), then k_path_bounce, which shades the hits,
+// writes the next segment in place and lists the paths that go on.  FP32 with
+// the operation order fixed, so every bounce reproduces the oracle's bit for
+// bit:
 //   miss      radiance = throughput * sky, the path ends;
 //   hit       throughput *= albedo (the nearest texel's colour, RGBA8 / 255 or
 //             RGBA32F; `untex` for untextured triangles and u8 textures);
@@ -47,33 +47,20 @@ __device__ __forceinline__ void path_albedo(const DevScene& sc, uint32_t prim, f
                      : VSR_LDG(reinterpret_cast<const float*>(sc.texels + off) + 4 * k + c);
 }
 
-__global__ void k_path_init(const float4* __restrict__ rays, unsigned long long n,
-                            float4* __restrict__ work, float* __restrict__ f,
-                            float* __restrict__ radiance, uint32_t* __restrict__ segments) {
-    const unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    work[2 * i] = VSR_LDG(rays + 2 * i);
-    work[2 * i + 1] = VSR_LDG(rays + 2 * i + 1);
-    f[3 * i] = 1.0f;
-    f[3 * i + 1] = 1.0f;
-    f[3 * i + 2] = 1.0f;
-    radiance[3 * i] = 0.0f;
-    radiance[3 * i + 1] = 0.0f;
-    radiance[3 * i + 2] = 0.0f;
-    if (segments) segments[i] = 0;
-}
-
-// Shading of segment k of every live path (f[3i] < 0 marks a finished path).
-__global__ void k_path_bounce(DevScene sc, PathDev pd, const float* __restrict__ verts,
-                              const uint32_t* __restrict__ idx, float4* __restrict__ work,
-                              const float4* __restrict__ hits, float* __restrict__ f,
-                              const float* __restrict__ dirs, uint32_t k,
-                              unsigned long long n, float* __restrict__ radiance,
-                              uint32_t* __restrict__ segments) {
-    const unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float fr = f[3 * i], fg = f[3 * i + 1], fb = f[3 * i + 2];
-    if (fr < 0.0f) return;
+// Segment k of path i: true when the path goes on, its next segment written.
+template <bool FIRST>
+__device__ __forceinline__ bool shade_segment(
+    const DevScene& sc, const PathDev& pd, const float* __restrict__ verts,
+    const uint32_t* __restrict__ idx, const float4* from, float4* work,
+    const float4* __restrict__ hits, float* __restrict__ f, const float* __restrict__ dirs,
+    uint32_t k, unsigned long long i, float* __restrict__ radiance,
+    uint32_t* __restrict__ segments) {
+    float fr = 1.0f, fg = 1.0f, fb = 1.0f;
+    if (!FIRST) {
+        fr = f[3 * i];
+        fg = f[3 * i + 1];
+        fb = f[3 * i + 2];
+    }
     if (segments) segments[i] = k + 1;
     const float4 h = VSR_LDG(hits + i);
     const uint32_t prim = __float_as_uint(h.w);
@@ -91,17 +78,17 @@ __global__ void k_path_bounce(DevScene sc, PathDev pd, const float* __restrict__
         fb = __fmul_rn(fb, alb[2]);
         done = k == pd.bounces;
     }
-    if (done) {
-        f[3 * i] = -1.0f;
-        work[2 * i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        work[2 * i + 1] = make_float4(0.0f, 0.0f, 1.0f, -1.0f);
-        return;
+    if (FIRST && prim != kMiss) {
+        radiance[3 * i] = 0.0f;
+        radiance[3 * i + 1] = 0.0f;
+        radiance[3 * i + 2] = 0.0f;
     }
+    if (done) return false;
     f[3 * i] = fr;
     f[3 * i + 1] = fg;
     f[3 * i + 2] = fb;
     // the next segment
-    const float4 ra = work[2 * i], rb = work[2 * i + 1];
+    const float4 ra = from[2 * i], rb = from[2 * i + 1];
     const float* a = verts + 3ull * VSR_LDG(idx + 3ull * prim);
     const float* b = verts + 3ull * VSR_LDG(idx + 3ull * prim + 1);
     const float* c = verts + 3ull * VSR_LDG(idx + 3ull * prim + 2);
@@ -142,131 +129,70 @@ __global__ void k_path_bounce(DevScene sc, PathDev pd, const float* __restrict__
                     __fmaf_rn(lx, t1y, __fmaf_rn(ly, t2y, __fmul_rn(lz, ny))),
                     __fmaf_rn(lx, t1z, __fmaf_rn(ly, t2z, __fmul_rn(lz, nz))),
                     __int_as_float(0x7f800000));
+    return !(fr < 0.0f);  // a negative throughput (red) ends the path
 }
 
-// Live-path compaction between bounces: a stable partition of the path
-// indices with the live paths (f[3i] >= 0) first, in index order, and the
-// finished ones after them.  The next segment's trace then takes ray perm[g]
-// in thread g, so live rays fill whole warps instead of sharing them with
-// finished paths, whose inactive rays end at the root box test.  Each ray is
-// traced exactly as before, so every result is unchanged.
-constexpr uint32_t kCompactThreads = 256;
+// Shading of segment k of the live paths, and the list of those that go on,
+// in one launch: `in` lists the live paths (*live_in of them), `out` and
+// *live_out (zero before the launch) receive the next segment's.  Each block
+// takes its run of `out` with one atomic, so paths stay together with their
+// neighbours; the order of the blocks, and so of the rays, does not change any
+// result.  Segment 0 (FIRST) has every path, its rays read from the caller's
+// buffer and throughput 1.  (The list was made by three further launches, a
+// count per block, one scan of the counts and a scatter, 13 us a bounce for
+// 518,400 paths, and finished paths went on as inactive rays.)
+constexpr uint32_t kBounceThreads = 256;
 
-__device__ __forceinline__ bool path_live(const float* __restrict__ f, unsigned long long i,
-                                          unsigned long long n) {
-    return i < n && f[3 * i] >= 0.0f;
-}
-
-// Number of live paths of this block before the thread's path, and the
-// block's live count in *total.  Every thread of the block calls it.
-__device__ __forceinline__ uint32_t block_live_rank(bool live, uint32_t* s_warp,
-                                                    uint32_t* total) {
+template <bool FIRST>
+__global__ void __launch_bounds__(kBounceThreads)
+    k_path_bounce(DevScene sc, PathDev pd, const float* __restrict__ verts,
+                  const uint32_t* __restrict__ idx, const float4* __restrict__ rays,
+                  float4* __restrict__ work, const float4* __restrict__ hits,
+                  float* __restrict__ f, const float* __restrict__ dirs, uint32_t k,
+                  unsigned long long n, const uint32_t* __restrict__ in,
+                  const uint32_t* __restrict__ live_in, uint32_t* __restrict__ out,
+                  uint32_t* __restrict__ live_out, float* __restrict__ radiance,
+                  uint32_t* __restrict__ segments) {
+    const unsigned long long g = (unsigned long long)blockIdx.x * kBounceThreads + threadIdx.x;
+    const unsigned long long limit = FIRST ? n : (unsigned long long)VSR_LDG(live_in);
+    if ((unsigned long long)blockIdx.x * kBounceThreads >= limit) return;  // the whole block
+    unsigned long long i = g;
+    bool live = false;
+    if (g < limit) {
+        if (!FIRST) i = VSR_LDG(in + g);
+        live = shade_segment<FIRST>(sc, pd, verts, idx, FIRST ? rays : work, work, hits, f, dirs, k,
+                                    i, radiance, segments);
+    }
+    if (k == pd.bounces) return;  // no next segment
+    __shared__ uint32_t s_warp[kBounceThreads / 32], s_base;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const unsigned b = __ballot_sync(kFullMask, live);
     if (lane == 0) s_warp[warp] = __popc(b);
     __syncthreads();
-    uint32_t before = 0, sum = 0;
-    for (uint32_t w = 0; w < kCompactThreads / 32u; ++w) {
+    uint32_t before = 0, total = 0;
+    for (uint32_t w = 0; w < kBounceThreads / 32u; ++w) {
         const uint32_t c = s_warp[w];
         if (w < warp) before += c;
-        sum += c;
+        total += c;
     }
-    *total = sum;
-    return before + __popc(b & ((1u << lane) - 1u));
-}
-
-__global__ void __launch_bounds__(kCompactThreads)
-    k_live_count(const float* __restrict__ f, unsigned long long n, uint32_t* __restrict__ counts) {
-    __shared__ uint32_t s_warp[kCompactThreads / 32];
-    const unsigned long long i = (unsigned long long)blockIdx.x * kCompactThreads + threadIdx.x;
-    uint32_t total = 0;
-    block_live_rank(path_live(f, i, n), s_warp, &total);
-    if (threadIdx.x == 0) counts[blockIdx.x] = total;
-}
-
-// Exclusive scan of the nb block counts in place, 1,024 at a time with a
-// running carry; counts[nb] receives the number of live paths.
-__global__ void __launch_bounds__(1024) k_live_scan(uint32_t* __restrict__ counts, uint32_t nb) {
-    __shared__ uint32_t s_warp[32];
-    __shared__ uint32_t s_carry;
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0) s_carry = 0;
+    if (threadIdx.x == 0) s_base = total ? atomicAdd(live_out, total) : 0u;
     __syncthreads();
-    for (uint32_t base = 0; base < nb; base += 1024u) {
-        const uint32_t j = base + threadIdx.x;
-        const uint32_t v = j < nb ? counts[j] : 0u;
-        uint32_t x = v;  // inclusive scan within the warp
-        for (uint32_t o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(kFullMask, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) s_warp[warp] = x;
-        __syncthreads();
-        if (warp == 0) {
-            uint32_t w = s_warp[lane];
-            for (uint32_t o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(kFullMask, w, o);
-                if (lane >= o) w += y;
-            }
-            s_warp[lane] = w;
-        }
-        __syncthreads();
-        const uint32_t excl = s_carry + (warp ? s_warp[warp - 1] : 0u) + x - v;
-        if (j < nb) counts[j] = excl;
-        __syncthreads();
-        if (threadIdx.x == 1023) s_carry = excl + v;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) counts[nb] = s_carry;
-}
-
-__global__ void __launch_bounds__(kCompactThreads)
-    k_live_scatter(const float* __restrict__ f, unsigned long long n,
-                   const uint32_t* __restrict__ offsets, uint32_t nb, uint32_t* __restrict__ perm) {
-    __shared__ uint32_t s_warp[kCompactThreads / 32];
-    const unsigned long long i = (unsigned long long)blockIdx.x * kCompactThreads + threadIdx.x;
-    const bool live = path_live(f, i, n);
-    uint32_t total = 0;
-    const uint32_t rank = block_live_rank(live, s_warp, &total);
-    if (i >= n) return;
-    const uint32_t live_before = offsets[blockIdx.x];
-    if (live) {
-        perm[live_before + rank] = (uint32_t)i;
-    } else {
-        // finished paths before this one: in earlier blocks, then in this one
-        const uint32_t dead_before = blockIdx.x * kCompactThreads - live_before;
-        perm[offsets[nb] + dead_before + (threadIdx.x - rank)] = (uint32_t)i;
-    }
+    if (live) out[s_base + before + __popc(b & ((1u << lane) - 1u))] = (uint32_t)i;
 }
 
 }  // namespace
 
-uint32_t path_compact_blocks(unsigned long long n) {
-    return (uint32_t)((n + kCompactThreads - 1) / kCompactThreads);
-}
-
-cudaError_t launch_path_compact(const float* f, unsigned long long n, uint32_t* counts,
-                                uint32_t* perm, cudaStream_t stream) {
-    const uint32_t nb = path_compact_blocks(n);
-    k_live_count<<<nb, kCompactThreads, 0, stream>>>(f, n, counts);
-    k_live_scan<<<1, 1024, 0, stream>>>(counts, nb);
-    k_live_scatter<<<nb, kCompactThreads, 0, stream>>>(f, n, counts, nb, perm);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_path_init(const float4* rays, unsigned long long n, float4* work, float* f,
-                             float* radiance, uint32_t* segments, cudaStream_t stream) {
-    k_path_init<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(rays, n, work, f, radiance,
-                                                                 segments);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_path_bounce(const DevScene& sc, const PathDev& pd, const float* verts,
-                               const uint32_t* idx, float4* work, const float4* hits, float* f,
-                               const float* dirs, uint32_t k, unsigned long long n,
-                               float* radiance, uint32_t* segments, cudaStream_t stream) {
-    k_path_bounce<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(
-        sc, pd, verts, idx, work, hits, f, dirs, k, n, radiance, segments);
+cudaError_t launch_path_bounce(const DevScene& sc, const PathDev& pd, const PathBuffers& p,
+                               uint32_t k, unsigned long long n, cudaStream_t stream) {
+    const unsigned grid = (unsigned)((n + kBounceThreads - 1) / kBounceThreads);
+    if (k == 0)
+        k_path_bounce<true><<<grid, kBounceThreads, 0, stream>>>(
+            sc, pd, p.verts, p.idx, p.rays, p.work, p.hits, p.f, p.dirs, k, n, nullptr, nullptr,
+            p.list[0], p.live, p.radiance, p.segments);
+    else
+        k_path_bounce<false><<<grid, kBounceThreads, 0, stream>>>(
+            sc, pd, p.verts, p.idx, nullptr, p.work, p.hits, p.f, p.dirs, k, n,
+            p.list[(k - 1) & 1], p.live + k - 1, p.list[k & 1], p.live + k, p.radiance, p.segments);
     return cudaGetLastError();
 }
 

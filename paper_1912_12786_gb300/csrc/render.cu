@@ -279,13 +279,16 @@ __global__ void __launch_bounds__(256) k_render_backward_hits(
 
 // Ambient-occlusion render: c = albedo_rgb(uv) * (1 - occluded / spp) for a
 // primary hit, background for a miss.  The closest-hit trace, the occlusion
-// rays traced any-hit and counted (the trace kernels; api.cu), then the
+// rays traced any-hit (the trace kernels; api.cu), then the count and the
 // shading of the saved hits here.
 
-// Shading of the saved hits; occ enters as the integer counts of
-// k_ao_count and leaves as the occluded fraction (0 for a miss).
+// Shading of the saved hits, with the occlusion rays' any-hit records counted
+// on the way (pixel i's at i * spp .. i * spp + spp - 1; integers, so the count
+// does not depend on the traversal order); occ receives the occluded fraction
+// (0 for a miss).
 __global__ void __launch_bounds__(256) k_ao_shade(DevScene sc, ShadeDev sh,
                                                   const float4* __restrict__ hits,
+                                                  const float4* __restrict__ ao_hits,
                                                   unsigned long long n, uint32_t spp,
                                                   float* __restrict__ occ,
                                                   float* __restrict__ image) {
@@ -296,7 +299,10 @@ __global__ void __launch_bounds__(256) k_ao_shade(DevScene sc, ShadeDev sh,
     float c[3] = {sh.bg[0], sh.bg[1], sh.bg[2]};
     float o = 0.0f;
     if (prim != kMiss) {
-        o = (float)reinterpret_cast<const uint32_t*>(occ)[i] / (float)spp;
+        uint32_t occluded = 0;
+        for (uint32_t k = 0; k < spp; ++k)
+            occluded += __float_as_uint(VSR_LDG(ao_hits + i * spp + k).w) != kMiss;
+        o = (float)occluded / (float)spp;
         const float vis = 1.0f - o;
         Bilinear b;
         albedo(sc, VSR_LDG(sc.geom + prim), lerp_uv(sc.uvs, prim, h.y, h.z), b);
@@ -373,8 +379,8 @@ cudaError_t render_align_error(unsigned* line) {
 
 cudaError_t launch_ao_shade(const DevScene& sc, const AoArgs& ao, unsigned long long n,
                             cudaStream_t stream) {
-    k_ao_shade<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(sc, ao.sh, ao.hits, n, ao.spp,
-                                                                ao.occ, ao.image);
+    k_ao_shade<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(sc, ao.sh, ao.hits, ao.ao_hits, n,
+                                                                ao.spp, ao.occ, ao.image);
     return cudaGetLastError();
 }
 

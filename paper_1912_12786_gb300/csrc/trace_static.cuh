@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(256) k_trace(DevScene sc, IsectParams ip,
                                                uint2* __restrict__ counters,
                                                uint4* __restrict__ stats) {
     extern __shared__ uint32_t s_stack[];
-    const unsigned long long g = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned long long g = slot_of_thread(map);
     if (g >= map.threads) return;
     const unsigned long long i = ray_of_thread(g, map);
     if (i >= map.n) return;
@@ -59,7 +59,7 @@ __device__ __forceinline__ void trace_ls(DevScene sc, IsectParams ip,
                                          uint4* __restrict__ stats,
                                          const DevScene* __restrict__ user) {
     extern __shared__ uint32_t s_stack[];
-    const unsigned long long g = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned long long g = slot_of_thread(map);
     const unsigned long long i = g < map.threads ? ray_of_thread(g, map) : map.n;
     bool busy = i < map.n;
     Ray r;
@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(256, MINB) k_trace_cap(DevScene sc, IsectParam
                                                          RayMap map, float4* __restrict__ hits,
                                                          uint2* __restrict__ counters) {
     extern __shared__ uint32_t s_stack[];
-    const unsigned long long g = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned long long g = slot_of_thread(map);
     if (g >= map.threads) return;
     const unsigned long long i = ray_of_thread(g, map);
     if (i >= map.n) return;

@@ -96,7 +96,7 @@ struct DevScene {
 // the image's right or bottom edge take no ray.  perm != null (coherence
 // order, width 0): thread g takes ray perm[g], a permutation of the rays
 // sorted by origin and direction.  Rays and hits keep the caller's layout in
-// every case.
+// every case.  A perm entry of kMiss names no ray.
 struct RayMap {
     unsigned long long n;        // rays
     unsigned long long threads;  // threads the grid covers
@@ -812,8 +812,9 @@ __host__ __device__ constexpr int min_blocks() {
 template <class H>
 __device__ __forceinline__ void isect_setup(H&, const IsectParams&, const DevScene*) {}
 
-// Sixteenths of a warp's busy lanes that end warp_step's node loop.
-constexpr uint32_t kLeafShare = 7u;
+// Passes waited per descending lane that end warp_step's node loop (4 to 10
+// differ by 1%).
+constexpr uint32_t kLeafWait = 6u;
 
 // One outer iteration of the while-while traversal (Section 3.2) run by the
 // whole warp in lock step: all 32 lanes call it, lanes without a ray with
@@ -825,20 +826,25 @@ constexpr uint32_t kLeafShare = 7u;
 // issuing on its own.)  Then every lane that has reached a leaf tests its
 // primitives, one per pass.
 //
-// The node loop ends when kLeafShare of the busy lanes have reached a leaf or
-// finished, not when the last lane has: on incoherent rays the number of inner
-// nodes between two leaves varies so much that the wait for the slowest of 32
-// lanes is about three times the mean (13 inner nodes per leaf, 200,000 random
-// quads), and the early end costs only leaf passes with fewer lanes.  Each
+// The node loop ends when the passes that lanes with a leaf (or without nodes)
+// have waited add up to kLeafWait per lane still descending -- about what a
+// leaf pass without those costs -- and not when the last lane has a leaf: on
+// incoherent rays the number of inner nodes between two leaves varies so much
+// that the wait for the slowest of 32 lanes is about three times the mean (13
+// inner nodes per leaf, 200,000 random quads), and the early end costs only
+// leaf passes with fewer lanes.  Where leaves follow each other closely (the
+// forest: 3.6 nodes per leaf) most lanes have one when the sum is reached.  Each
 // lane still visits its own nodes and leaves in the order of traverse_body;
 // only how the warp interleaves them differs.  Measured against a node loop
 // that ran until every lane held a leaf while lanes with one went on
 // speculatively (the speculative traversal of Aila and Laine, 2009, with the
 // bookkeeping that undoes what the leaf culls), persistent, 1,000,003 diffuse
-// rays on 200,000 triangles, alpha texture: closest hit 1,148 -> 838 us, any
+// rays on 200,000 triangles, alpha texture: closest hit 1,148 -> 835 us, any
 // hit 1,011 -> 812 us, 15.8 of 32 lanes active; 1.2 M occlusion rays on 2 M
-// triangles 533 -> 505 us.  The share is flat between 3/8 and 5/8 (838-850
-// us) and loses on both sides (1/8: 952, 7/8: 977 us).
+// triangles 533 -> 496 us.  A fixed share of the lanes in place of the sum does
+// as well on random quads (flat from 3/8 to 5/8 of the lanes, 838-850 us) but
+// not on path segments through the forest (1,305 against 1,249 us a frame).
+// Two to four nodes per vote instead of one: 866-885 us.
 // Returns true on busy lanes whose ray has finished (result in best).
 template <int Q, class H, bool STATS, class B, class S>
 __device__ __forceinline__ bool warp_step(const DevScene& sc, const IsectParams& ip,
@@ -846,46 +852,41 @@ __device__ __forceinline__ bool warp_step(const DevScene& sc, const IsectParams&
                                           uint32_t& ref, uint32_t& steps, S& stk) {
     bool done = false;
     const uint32_t held = (uint32_t)__popc(__ballot_sync(kFullMask, busy));
-    const uint32_t share = held * kLeafShare / 16u + 1u;
+    uint32_t waited = 0;
     for (;;) {
         const bool inner = busy && !done && !(ref & kLeafBit);
         const uint32_t descending = (uint32_t)__popc(__ballot_sync(kFullMask, inner));
-        if (descending == 0u || descending + share <= held) break;
+        waited += held - descending;
+        if (waited >= kLeafWait * descending) break;
         if (inner) {
-            if (++steps > sc.max_steps) {
-                atomicOr(sc.err, kErrSteps);
-                best.fail();
-                done = true;
-            } else {
-                const float4* p = sc.nodes + 4ull * (ref >> 2);
-                float4 la, lb, ra, rb;
-                load_pair(p, la, lb, ra, rb);
-                const float tfar = h.far((Q == kClosest) ? best.t : r.tmax);
-                h.box();
-                h.box();
-                if (STATS) st.boxes += 2;
-                const bool hl = box_hit(r, la, lb, tfar) && h.keep(ip, la, lb);
-                const bool hr = box_hit(r, ra, rb, tfar) && h.keep(ip, ra, rb);
-                const uint32_t rl = __float_as_uint(la.w), rr = __float_as_uint(ra.w);
-                if (hl && hr) {
-                    const bool neg = (r.negmask >> (ref & 3u)) & 1u;
-                    if (stk.n >= sc.stack_depth) {
-                        atomicOr(sc.err, kErrStack);
-                        best.fail();
-                        done = true;
-                    } else {
-                        stk.push(neg ? rl : rr);
-                        ref = neg ? rr : rl;
-                    }
-                } else if (hl) {
-                    ref = rl;
-                } else if (hr) {
-                    ref = rr;
-                } else if (stk.n) {
-                    ref = stk.pop();
-                } else {
+            const float4* p = sc.nodes + 4ull * (ref >> 2);
+            float4 la, lb, ra, rb;
+            load_pair(p, la, lb, ra, rb);
+            const float tfar = h.far((Q == kClosest) ? best.t : r.tmax);
+            h.box();
+            h.box();
+            if (STATS) st.boxes += 2;
+            const bool hl = box_hit(r, la, lb, tfar) && h.keep(ip, la, lb);
+            const bool hr = box_hit(r, ra, rb, tfar) && h.keep(ip, ra, rb);
+            const uint32_t rl = __float_as_uint(la.w), rr = __float_as_uint(ra.w);
+            if (hl && hr) {
+                const bool neg = (r.negmask >> (ref & 3u)) & 1u;
+                if (stk.n >= sc.stack_depth) {
+                    atomicOr(sc.err, kErrStack);
+                    best.fail();
                     done = true;
+                } else {
+                    stk.push(neg ? rl : rr);
+                    ref = neg ? rr : rl;
                 }
+            } else if (hl) {
+                ref = rl;
+            } else if (hr) {
+                ref = rr;
+            } else if (stk.n) {
+                ref = stk.pop();
+            } else {
+                done = true;
             }
         }
     }

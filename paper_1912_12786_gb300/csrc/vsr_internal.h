@@ -163,25 +163,31 @@ cudaError_t launch_instances(const InstLaunch& L, int kind, int query, bool dyna
 // (0 if none), cleared after reading.
 cudaError_t instances_align_error(unsigned* line);
 
-// Diffuse path tracing (path.cu): shading and the next segment per bounce.
+// Diffuse path tracing (path.cu): shading, the next segment and the list of
+// live paths per bounce.
 struct PathDev {
     uint32_t bounces;
     float eps;
     float sky[3];
     float untex[3];
 };
-cudaError_t launch_path_init(const float4* rays, unsigned long long n, float4* work, float* f,
-                             float* radiance, uint32_t* segments, cudaStream_t stream);
-cudaError_t launch_path_bounce(const DevScene& sc, const PathDev& pd, const float* verts,
-                               const uint32_t* idx, float4* work, const float4* hits, float* f,
-                               const float* dirs, uint32_t k, unsigned long long n,
-                               float* radiance, uint32_t* segments, cudaStream_t stream);
-// Live-path compaction (path.cu): perm[0..n) becomes the path indices with
-// the live paths first, in index order; counts holds path_compact_blocks(n)
-// + 1 words of scratch.  n < 2^32.
-uint32_t path_compact_blocks(unsigned long long n);
-cudaError_t launch_path_compact(const float* f, unsigned long long n, uint32_t* counts,
-                                uint32_t* perm, cudaStream_t stream);
+// The caller's arrays and the scratch of a path-traced frame.  list[k & 1] and
+// live[k] receive the paths that segment k + 1 traces (live zeroed before).
+struct PathBuffers {
+    const float* verts;
+    const uint32_t* idx;
+    const float4* rays;
+    const float* dirs;
+    float* radiance;
+    uint32_t* segments;
+    float4* work;  // the next segments
+    float4* hits;
+    float* f;      // throughputs
+    uint32_t* list[2];
+    uint32_t* live;
+};
+cudaError_t launch_path_bounce(const DevScene& sc, const PathDev& pd, const PathBuffers& p,
+                               uint32_t k, unsigned long long n, cudaStream_t stream);
 // Source line of the first misaligned load the path kernels skipped (0 if
 // none), cleared after reading.
 cudaError_t path_align_error(unsigned* line);
@@ -276,12 +282,13 @@ struct AoArgs {
     const float2* xi;
     float tmax, eps;
     float4* hits;        // primary closest hits (written by the trace, read after)
-    float* occ;          // occlusion counts (zeroed uint32), then occluded fractions
+    float* occ;          // occluded fractions
     float* image;        // forward
     const float* g;      // backward
     float* grad_texels;  // backward
+    const float4* ao_hits = nullptr;  // forward: the occlusion rays' any-hit records
 };
-// Image and occluded fractions from the hits and counts.
+// Image and occluded fractions from the hits and the occlusion records.
 cudaError_t launch_ao_shade(const DevScene& sc, const AoArgs& ao, unsigned long long n,
                             cudaStream_t stream);
 // Texel gradients from the saved hits and occluded fractions.

@@ -75,10 +75,9 @@ namespace vsr {
 constexpr uint32_t kLeft = 0x20000000u, kRight = 0x40000000u;
 constexpr uint32_t kRecField = 0x1FFFFFC0u;  // record << 6
 constexpr uint32_t kWideSlack = 2u;
-// Sixteenths of a warp's busy lanes that end wide_step's node loop (closest /
-// any / occlusion us above: 4: 838 / 742 / 457, 7: 786 / 705 / 428, 9: 785 /
-// 711 / 424, 11: 812 / 738 / 420).
-constexpr uint32_t kWideShare = 8u;
+// As kLeafWait for wide_step, whose passes make two levels (2 to 5 differ by
+// 1%).
+constexpr uint32_t kWideWait = 4u;
 
 typedef unsigned long long f32x2;  // two floats, the first in the low word
 
@@ -324,11 +323,12 @@ __device__ __forceinline__ bool wide_step(const DevScene& sc, const IsectParams&
                                           WideLane<Q, H>& w, const LaneStore& m, bool busy) {
     bool live = busy;
     const uint32_t held = (uint32_t)__popc(__ballot_sync(kFullMask, busy));
-    const uint32_t share = held * kWideShare / 16u + 1u;
+    uint32_t waited = 0;
     for (;;) {
         const bool inner = live && !(w.ref & kLeafBit);
         const uint32_t descending = (uint32_t)__popc(__ballot_sync(kFullMask, inner));
-        if (descending == 0u || descending + share <= held) break;
+        waited += held - descending;
+        if (waited >= kWideWait * descending) break;
         if (inner) live = w.visit(sc, m);
     }
     // test the leaves reached, one primitive of every lane per pass
