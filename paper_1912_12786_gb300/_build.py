@@ -23,7 +23,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CU_SOURCES = ["api.cu", "trace_static.cu", "trace_k0.cu", "trace_k1.cu", "trace_k2.cu",
               "trace_k4.cu", "trace_k8.cu", "trace_oct.cu", "trace_caps.cu", "trace_dynamic.cu", "trace_multi.cu",
               "trace_instances.cu", "render.cu", "batch.cu", "sort.cu", "path.cu", "measure.cu",
-              "refit.cu", "wide.cu", "trace_wide.cu"]
+              "refit.cu", "wide.cu", "trace_wide.cu", "scratch.cu"]
 CPP_SOURCES = [os.path.join(PKG, "inputs", "bvh_build.cpp")]
 _lock = threading.Lock()
 

@@ -32,6 +32,7 @@ struct vsr_scene {
     float4* d_tris = nullptr;
     uint32_t num_nodes = 0, max_depth = 0;
     bool has_bvh = false;
+    bool pooled = false;  // counted by the scratch pool
     DevScene dev{};
     DevScene* d_user = nullptr;
     uint32_t* d_err = nullptr;  // [0] device error word; [1] refit box state
@@ -433,7 +434,7 @@ cudaError_t launch_ordered(LaunchArgs a, int kind, bool dynamic) {
     if (a.n > coherence_sort_max_rays()) return cudaErrorInvalidValue;
     uint32_t* scratch = nullptr;
     const uint32_t ntiles = (uint32_t)((a.n + kSortTileRays - 1) / kSortTileRays);
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&scratch),
+    cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&scratch),
                                     coherence_sort_words((uint32_t)a.n, ntiles) * sizeof(uint32_t),
                                     a.stream);
     if (e != cudaSuccess) return e;
@@ -525,6 +526,7 @@ vsr_status tune_trace(vsr_scene* s, const LaunchArgs& base, const vsr_intersecto
                 c.persistent = 1u;
                 c.refill_threshold = r;
                 c.lockstep = ls;
+                if (ls) c.stack_regs = 0u;  // the two-level records take no others
                 consider(c);
             }
     }
@@ -625,6 +627,8 @@ vsr_status vsr_scene_create_indexed(const float* verts, uint32_t nverts, const u
             return bail(cuda_fail(e, "texture upload"));
     }
     s->h_tex = td;
+    scratch_scene_created();
+    s->pooled = true;
     *out = s;
     return VSR_OK;
 }
@@ -653,6 +657,7 @@ vsr_status vsr_scene_destroy(vsr_scene* s) {
     dfree(s->d_texels);
     dfree(s->d_user);
     dfree(s->d_err);
+    if (s->pooled) scratch_scene_destroyed();
     delete s;
     return VSR_OK;
 }
@@ -1086,7 +1091,7 @@ extern "C" vsr_status vsr_render(vsr_scene* s, const vsr_ray* rays, uint64_t n,
     // shading pass from the records
     float4* h = reinterpret_cast<float4*>(hits);
     cudaError_t e = cudaSuccess;
-    if (!h) e = cudaMallocAsync(reinterpret_cast<void**>(&h), n * sizeof(float4), a.stream);
+    if (!h) e = scratch_alloc(reinterpret_cast<void**>(&h), n * sizeof(float4), a.stream);
     if (e != cudaSuccess) return cuda_fail(e, "render scratch");
     a.hits = h;
     e = launch_static(a, is->kind, false);
@@ -1127,7 +1132,7 @@ extern "C" vsr_status vsr_trace_backward(vsr_scene* s, const vsr_ray* rays, uint
     // the closest hits traced again into stream-ordered scratch, then the
     // adjoint from them
     float4* h = nullptr;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&h), n * sizeof(float4), a.stream);
+    cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&h), n * sizeof(float4), a.stream);
     if (e != cudaSuccess) return cuda_fail(e, "backward scratch");
     a.hits = h;
     e = launch_static(a, is->kind, false);
@@ -1228,7 +1233,7 @@ extern "C" vsr_status vsr_render_ao(vsr_scene* s, const vsr_ray* rays, uint64_t 
     // and the any-hit query, else the default
     const uint64_t m = n * spp;
     uint8_t* scratch = nullptr;
-    e = cudaMallocAsync(reinterpret_cast<void**>(&scratch), m * 48 + 16, a.stream);
+    e = scratch_alloc(reinterpret_cast<void**>(&scratch), m * 48 + 16, a.stream);
     if (e != cudaSuccess) return cuda_fail(e, "ao occlusion");
     float4* ao_rays = reinterpret_cast<float4*>(scratch);
     float4* ao_hits = ao_rays + 2 * m;
@@ -1355,22 +1360,12 @@ extern "C" vsr_status vsr_scene_update(vsr_scene* s, const float* verts, uint32_
 // on the counter.  The counter is cleared on the caller's stream before each
 // launch.
 
-namespace {
-
-constexpr unsigned kNoallocWords = 32;  // 256 bytes
-constexpr unsigned kNoallocWordsPerCall = 1;
-// the limit of any single launch here: (2^31 - 2) * 32 rays
-constexpr uint64_t kNoallocMaxRays = (uint64_t)(std::numeric_limits<int>::max() - 1) * 32ull;
-static_assert(kNoallocWordsPerCall <= kNoallocWords, "scratch array too small");
-
-static __device__ __align__(256) unsigned long long g_noalloc_scratch[kNoallocWords];
-
 typedef int (*CtxGetCurrentFn)(void** ctx);
 typedef int (*CtxGetIdFn)(void* ctx, unsigned long long* id);
 
 // Unique id of the calling thread's current CUDA context (ids are never
 // reused within a process), read through the driver's entry points.
-bool current_context_id(unsigned long long* id) {
+bool vsr::current_context_id(unsigned long long* id) {
     static CtxGetCurrentFn get_current = nullptr;
     static CtxGetIdFn get_id = nullptr;
     static std::once_flag once;
@@ -1392,6 +1387,16 @@ bool current_context_id(unsigned long long* id) {
     if (!get_current || !get_id || get_current(&ctx) != 0 || !ctx) return false;
     return get_id(ctx, id) == 0;
 }
+
+namespace {
+
+constexpr unsigned kNoallocWords = 32;  // 256 bytes
+constexpr unsigned kNoallocWordsPerCall = 1;
+// the limit of any single launch here: (2^31 - 2) * 32 rays
+constexpr uint64_t kNoallocMaxRays = (uint64_t)(std::numeric_limits<int>::max() - 1) * 32ull;
+static_assert(kNoallocWordsPerCall <= kNoallocWords, "scratch array too small");
+
+static __device__ __align__(256) unsigned long long g_noalloc_scratch[kNoallocWords];
 
 constexpr int kNoallocMaxDevices = 64;
 std::mutex g_noalloc_mutex;
@@ -2183,7 +2188,7 @@ extern "C" vsr_status vsr_path_trace(vsr_scene* s, const vsr_ray* rays, uint64_t
                    at_live = (at_list + 8 * m + 15) & ~15ull, at_work = at_live + 4 * 64,
                    bytes = at_work + 8;
     uint8_t* scratch = nullptr;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&scratch), bytes, cs);
+    cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&scratch), bytes, cs);
     if (e == cudaSuccess) e = cudaMemsetAsync(scratch + at_live, 0, 4 * 64, cs);
     PathBuffers b{};
     b.verts = s->d_verts;

@@ -101,6 +101,15 @@ inline unsigned long long spread_rays(RayMap& map, unsigned warps_per_sm) {
     return ((map.threads + (1ull << map.lane_bits) - 1) >> map.lane_bits) * 32ull;
 }
 
+// Stream-ordered scratch (scratch.cu), freed with cudaFreeAsync.  The pool lives
+// while scenes do; both notes are for the current device.
+cudaError_t scratch_alloc(void** ptr, size_t bytes, cudaStream_t stream);
+void scratch_scene_created();
+void scratch_scene_destroyed();
+// Unique id of the calling thread's current CUDA context (ids are never reused
+// within a process).
+bool current_context_id(unsigned long long* id);
+
 // Run `launch(counter)` with a persistent launch's ray counter, zeroed on
 // `stream` first: `given` when not null, else 8 bytes of stream-ordered
 // scratch freed on the stream after the launch, so persistent launches on
@@ -110,7 +119,7 @@ cudaError_t with_ray_counter(unsigned long long* given, cudaStream_t stream, Lau
     unsigned long long* work = given;
     cudaError_t e = cudaSuccess;
     if (!work) {
-        e = cudaMallocAsync(reinterpret_cast<void**>(&work), sizeof(unsigned long long), stream);
+        e = scratch_alloc(reinterpret_cast<void**>(&work), sizeof(unsigned long long), stream);
         if (e != cudaSuccess) return e;
     }
     e = cudaMemsetAsync(work, 0, sizeof(unsigned long long), stream);
