@@ -135,8 +135,8 @@ __global__ void __launch_bounds__(256) k_trace_inst(InstDev is, IsectParams ip,
                 // descent ends by construction (children follow their parent)
                 while (!(ref & kLeafBit)) {
                     const float4* p = is.nodes + 4ull * (ref >> 2);
-                    const float4 la = VSR_LDG(p), lb = VSR_LDG(p + 1), qa = VSR_LDG(p + 2),
-                                 qb = VSR_LDG(p + 3);
+                    float4 la, lb, qa, qb;
+                    load_pair(p, la, lb, qa, qb);
                     const float tfar = (Q == kClosest) ? best.t : r.tmax;
                     h.box();
                     h.box();
@@ -250,8 +250,8 @@ struct InstWalk {
         // descent ends by construction (children follow their parent)
         while (!(tref & kLeafBit)) {
             const float4* p = is.nodes + 4ull * (tref >> 2);
-            const float4 la = VSR_LDG(p), lb = VSR_LDG(p + 1), qa = VSR_LDG(p + 2),
-                         qb = VSR_LDG(p + 3);
+            float4 la, lb, qa, qb;
+            load_pair(p, la, lb, qa, qb);
             const float tfar = (Q == kClosest) ? best.t : r.tmax;
             h.box();
             h.box();

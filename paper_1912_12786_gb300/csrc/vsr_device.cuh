@@ -169,15 +169,17 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
 // The two children of an inner node: a 64-byte aligned pair of 32-byte
 // records, read as two 256-bit loads (the address is 32-byte aligned by
 // construction: the node array comes from cudaMalloc and pair k sits at byte
-// 64 k).  Checked builds read them as four checked 128-bit loads.
+// 64 k).  Checked builds check the pair's address once.  (Four checked 128-bit
+// loads cost a test and a branch each.)
 __device__ __forceinline__ void load_pair(const float4* p, float4& la, float4& lb, float4& ra,
                                           float4& rb) {
 #ifdef VSR_CHECKED_LOADS
-    la = VSR_LDG(p);
-    lb = VSR_LDG(p + 1);
-    ra = VSR_LDG(p + 2);
-    rb = VSR_LDG(p + 3);
-#else
+    if (reinterpret_cast<unsigned long long>(p) % 64u) {
+        atomicCAS(&g_vsr_align_line, 0u, (unsigned)__LINE__);
+        la = lb = ra = rb = make_float4(0.0f, 0.0f, 0.0f, __uint_as_float(kLeafBit));
+        return;
+    }
+#endif
     asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
         : "=f"(la.x), "=f"(la.y), "=f"(la.z), "=f"(la.w), "=f"(lb.x), "=f"(lb.y), "=f"(lb.z),
           "=f"(lb.w)
@@ -186,7 +188,6 @@ __device__ __forceinline__ void load_pair(const float4* p, float4& la, float4& l
         : "=f"(ra.x), "=f"(ra.y), "=f"(ra.z), "=f"(ra.w), "=f"(rb.x), "=f"(rb.y), "=f"(rb.z),
           "=f"(rb.w)
         : "l"(p + 2));
-#endif
 }
 
 __device__ __forceinline__ float guard_dir(float d) {
