@@ -216,7 +216,11 @@ typedef struct vsr_trace_params {
                                   node loop ends when the lanes that reached a
                                   leaf have waited long enough, and they test
                                   their leaves together.
-                                  0 = each lane runs its own loops.  Each ray
+                                  0 = each lane runs its own loops (static
+                                  launches of one ray per thread with
+                                  stack_regs, octant and reg_cap_blocks 0 may
+                                  run in lock step on trees where that is
+                                  faster).  Each ray
                                   visits the same nodes and leaves in the same
                                   order either way, so results are identical.
                                   vsr_trace and vsr_path_trace (static or

@@ -31,6 +31,7 @@ struct vsr_scene {
     uint32_t* d_wide = nullptr;  // two-level node records; null: the binary nodes are walked
     float4* d_tris = nullptr;
     uint32_t num_nodes = 0, max_depth = 0;
+    uint64_t records_up_to = 0;  // records_limit of the tree
     bool has_bvh = false;
     bool pooled = false;  // counted by the scratch pool
     DevScene dev{};
@@ -285,6 +286,36 @@ void free_bvh(vsr_scene* s) {
     s->has_bvh = false;
 }
 
+// Up to how many rays a static launch of one ray per thread that leaves the
+// traversal's form open runs in lock step over the records.  That pays where a
+// ray descends through many boxes per leaf, because lanes then reach their
+// leaves far apart even when neighbouring rays agree; the surface areas of the
+// boxes tell, relative to the root's the expected visits of a ray that crosses
+// the scene: `inner` nodes, and inner per leaf.  Closest hit, alpha texture, us
+// per-lane / lock step, camera rays 480 x 270, 960 x 540 and 1920 x 1080 and
+// 1,000,000 diffuse rays:
+//   random quads, 2,000,000 (inner 291, 36 per leaf)
+//                           490/301  559/407  1373/1065  2789/2234
+//   random quads, 200,000 (149, 18)  209/146  252/215  549/565  1406/1262
+//   random quads, 50,000 (101, 13)   161/121  155/159  318/381  1038/997
+//   random quads, 4,096 (49, 6.8)     76/75    76/96  137/202   650/710
+//   sphere, 64,980 (33, 11)          120/118  147/160  244/320   734/727
+//   forest, 200,002 (304, 2.2)       113/137  152/245  405/705  2405/2561
+uint64_t records_limit(const vsr_bvh_node* nodes, uint32_t num_nodes) {
+    double inner = 0.0, leaf = 0.0, root = 0.0;
+    for (uint32_t i = 0; i < num_nodes; ++i) {
+        if (i == 1) continue;  // padding beside the root
+        const vsr_bvh_node& n = nodes[i];
+        const double x = (double)n.hi[0] - n.lo[0], y = (double)n.hi[1] - n.lo[1],
+                     z = (double)n.hi[2] - n.lo[2], a = x * y + y * z + z * x;
+        (n.count_axis >> 2 ? leaf : inner) += a;
+        if (i == 0) root = a;
+    }
+    if (!(root > 0.0) || !(inner >= 12.0 * leaf)) return 0;
+    const double visits = inner / root;
+    return visits >= 90.0 ? (uint64_t)std::min(32.0 * visits * visits, 1e15) : 0;
+}
+
 vsr_status validate_isect(const vsr_intersector* is, int32_t query) {
     if (!is) return fail(VSR_ERR_ARG, "intersector is null");
     if (is->kind < VSR_ISECT_NONE || is->kind > VSR_ISECT_CLIP)
@@ -423,6 +454,7 @@ vsr_status prepare_launch(vsr_scene* s, const vsr_ray* rays, uint64_t n,
     a.query = query;
     a.work = nullptr;  // persistent launches take their own counter
     a.dyn_user = s->d_user;
+    a.records_up_to = s->records_up_to;
     return VSR_OK;
 }
 
@@ -735,6 +767,7 @@ vsr_status vsr_bvh_load(vsr_scene* s, const void* blob, size_t bytes) {
     }
     s->num_nodes = num_nodes;
     s->max_depth = max_depth;
+    s->records_up_to = records_limit(nodes, num_nodes);
     DevScene& d = s->dev;
     d.nodes = s->d_nodes;
     d.tris = s->d_tris;

@@ -21,6 +21,12 @@ cudaError_t launch_static(const LaunchArgs& a, int kind, bool stats) {
     if (stats) return launch_static_k0(a, kind, true);
     if (a.reg_cap >= 3) return launch_static_capped(a, kind, a.reg_cap);
     if (walks_records(a, kind)) return launch_wide(a, kind);
+    // a shape that leaves the traversal's form open (records_limit, api.cu)
+    if (!a.persistent && !a.lockstep && !a.octant && a.reg_cap == 0 && a.n <= a.records_up_to) {
+        LaunchArgs b = a;
+        b.lockstep = 1u;
+        if (walks_records(b, kind)) return launch_wide(b, kind);
+    }
     // the octant-dispatching kernel also runs the launches that do not ask for
     // it (trace_oct.cu)
     if (a.octant || (!a.persistent && !a.lockstep && a.stack_regs == 0))

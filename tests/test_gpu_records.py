@@ -141,3 +141,27 @@ def test_records_after_refit_and_in_a_batch(V):
     _same(V, s, d * 1e12, "alpha_tex", "closest", "out of range")
     V.vsr_batch_destroy(b)
     s.close()
+
+
+@pytest.mark.parametrize("n_quads,n", [(25_000, 5000), (25_000, 700_001), (400, 5000)])
+def test_open_launches_match_binary(V, n_quads, n):
+    """Launches that leave the traversal's form open, on a tree with long
+    descents below and above the ray count at which they walk the records, and
+    on a shallow one: the records of the measurement kernel, which walks the
+    binary nodes."""
+    rng = np.random.default_rng(n_quads)
+    side = 0.08 * (2048 / n_quads) ** 0.5
+    v, i, uv = scenes._quads_to_tris(scenes.random_quads(rng, n_quads, 0, 1, 0.2 * side, side))
+    sc = scenes.Scene("quads", v, i, uv, np.zeros(len(i), np.uint32), [scenes.disc_alpha_u8()])
+    s = V.scene_from_inputs(sc, sc.bvh())
+    d = torch.from_numpy(scenes.diffuse_rays(rng, sc, n)).cuda()
+    stats = torch.empty(n, 4, device="cuda", dtype=torch.int32)
+    for kind in ("default", "alpha_tex", "proc_alpha"):
+        for query in ("closest", "any"):
+            want = torch.empty(n, 4, device="cuda")
+            got = torch.full_like(want, 7.0)
+            V.vsr_trace_stats(s, d, V.intersector(kind), query, want, stats)
+            V.vsr_trace(s, d, V.intersector(kind), query, got, None, V.trace_params())
+            assert torch.equal(got.view(torch.int32), want.view(torch.int32)), (kind, query)
+    assert V.vsr_get_device_error(s) == 0
+    s.close()
