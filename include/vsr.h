@@ -392,8 +392,9 @@ vsr_status vsr_trace_multi(vsr_scene* scene, const vsr_ray* rays, uint64_t n,
  *   radiance  device float32 [n * 3], written
  *   segments  device uint32 [n] or NULL: closest-hit queries path i made
  *   params    every segment's launch; image_width maps the primary
- *             segments to pixel tiles; persistent launches, lock step and
- *             the octant box test apply to each segment depth; ray_order 0
+ *             segments to pixel tiles; persistent launches and lock step
+ *             apply to each segment depth (with neither, segments after a
+ *             bounce may use them); ray_order 0
  * One closest-hit launch per segment depth plus one shading launch, on
  * `stream`.  The shading launch also lists the paths that go on (their order
  * may vary from run to run; results do not depend on it), and the next

@@ -458,6 +458,28 @@ vsr_status prepare_launch(vsr_scene* s, const vsr_ray* rays, uint64_t n,
     return VSR_OK;
 }
 
+// The launch of path segments after a bounce, whose rays point anywhere, where
+// the caller left the shape at one ray per thread with per-lane loops: 7 of 32
+// lanes are active then.  Lock step on the binary nodes, persistent from three
+// waves of resident threads on -- unless the tree is one for the records
+// (records_limit), which launch_static sees to.  us a frame per-lane / lock step
+// / persistent: forest 1920 x 1080, 3 bounces 4,460 / 4,116 / 3,775; 960 x 540
+// 1,263 / 1,194 / 1,132; 514 x 298, 2 bounces 469 / 449 / 481; random quads
+// (4,000) 800 x 500 329 / 318 / 338; the records' tree (200,000 quads) 837 / 883 /
+// 914.
+void bounce_launch(LaunchArgs& a) {
+    if (a.persistent || a.lockstep || a.stack_regs || a.reg_cap || a.n <= a.records_up_to) return;
+    a.lockstep = 1u;
+    a.octant = 0u;
+    a.binary_nodes = true;
+    if (a.n >= 3ull * 1024ull * (unsigned)sm_count()) {
+        a.persistent = 1u;
+        a.block = 64u;
+        a.refill = 24u;
+        a.blocks_per_sm = 0u;
+    }
+}
+
 // Launch `a` in the rays' coherence order (vsr_trace with ray_order 1):
 // scratch from the stream-ordered allocator, the sort of the rays by origin
 // and direction, the trace through the resulting permutation, the scratch
@@ -2243,6 +2265,7 @@ extern "C" vsr_status vsr_path_trace(vsr_scene* s, const vsr_ray* rays, uint64_t
     for (uint32_t k = 0; e == cudaSuccess && k <= pp->bounces; ++k) {
         if (k == 1) {
             a.rays = b.work;
+            if (is->dispatch == VSR_DISPATCH_STATIC) bounce_launch(a);
         }
         if (k > 0) {
             a.map = RayMap{n, n, 0u, 0u, b.list[(k - 1) & 1]};

@@ -90,7 +90,7 @@ cudaError_t wide_kind(const LaunchArgs& a, int kind) {
 }  // namespace
 
 bool walks_records(const LaunchArgs& a, int kind) {
-    return a.sc.wide && kind >= 0 && kind <= 3 && a.lockstep && a.stack_regs == 0;
+    return a.sc.wide && !a.binary_nodes && kind >= 0 && kind <= 3 && a.lockstep && a.stack_regs == 0;
 }
 
 cudaError_t launch_wide(const LaunchArgs& a, int kind) {

@@ -33,6 +33,7 @@ struct LaunchArgs {
     uint32_t reg_cap;          // 0: each kernel's own register budget; 1, 3..6:
                                // __launch_bounds__(256, reg_cap) variants
     uint32_t lockstep = 0;     // 1: the warp runs the traversal in lock step
+    bool binary_nodes = false;   // lock step on the binary nodes, not the records
     uint64_t records_up_to = 0;  // rays up to which a launch that leaves the form
                                  // open walks the records in lock step
     uint32_t octant = 0;       // 1: box tests specialised to a warp's shared
