@@ -23,8 +23,7 @@ struct vsr_scene {
     uint32_t ntri = 0, nverts = 0, ntex = 0;
     float* d_verts = nullptr;
     uint32_t* d_idx = nullptr;
-    float2* d_uvs = nullptr;
-    uint32_t* d_geom = nullptr;
+    float4* d_attrs = nullptr;
     TexDesc* d_tex = nullptr;
     uint8_t* d_texels = nullptr;
     float4* d_nodes = nullptr;
@@ -226,6 +225,17 @@ __global__ void k_build_tris(const float* __restrict__ verts, const uint32_t* __
         make_float4(__fsub_rn(b[0], a[0]), __fsub_rn(b[1], a[1]), __fsub_rn(b[2], a[2]), 0.0f);
     tris[3ull * s + 2] =
         make_float4(__fsub_rn(c[0], a[0]), __fsub_rn(c[1], a[1]), __fsub_rn(c[2], a[2]), 0.0f);
+}
+
+// 24 + 4 bytes in separate arrays took an alpha test three sectors and one
+// round trip more (the texture id first): see alpha_tex_accept.
+__global__ void k_pack_attrs(const float2* __restrict__ uvs, const uint32_t* __restrict__ geom,
+                             uint32_t n, float4* __restrict__ attrs) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const float2 c0 = uvs[3ull * i], c1 = uvs[3ull * i + 1], c2 = uvs[3ull * i + 2];
+    attrs[2ull * i] = make_float4(c0.x, c0.y, c1.x, c1.y);
+    attrs[2ull * i + 1] = make_float4(c2.x, c2.y, __uint_as_float(geom[i]), 0.0f);
 }
 
 __global__ void k_shadow_rays(const float4* __restrict__ rays, const float4* __restrict__ hits,
@@ -619,6 +629,26 @@ int32_t vsr_version(void) { return 100; }
 
 const char* vsr_last_error(void) { return g_err.c_str(); }
 
+// Interleaves the texture coordinates and texture ids on the device.
+static cudaError_t upload_attrs(float4* attrs, const float* uvs, const uint32_t* geom_id,
+                                uint32_t ntri) {
+    float2* d_uvs = nullptr;
+    uint32_t* d_geom = nullptr;
+    cudaError_t e = dmalloc(&d_uvs, 3ull * ntri);
+    if (e == cudaSuccess) e = dmalloc(&d_geom, (size_t)ntri);
+    if (e == cudaSuccess) e = cudaMemcpy(d_uvs, uvs, 24ull * ntri, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(d_geom, geom_id, 4ull * ntri, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) {
+        k_pack_attrs<<<(ntri + 255u) / 256u, 256>>>(d_uvs, d_geom, ntri, attrs);
+        e = cudaGetLastError();
+        const cudaError_t s = cudaStreamSynchronize(nullptr);
+        if (e == cudaSuccess) e = s;
+    }
+    dfree(d_uvs);
+    dfree(d_geom);
+    return e;
+}
+
 vsr_status vsr_scene_create_indexed(const float* verts, uint32_t nverts, const uint32_t* idx,
                                     const float* uvs, const uint32_t* geom_id, uint32_t ntri,
                                     const vsr_texture_desc* tex, uint32_t ntex,
@@ -660,16 +690,14 @@ vsr_status vsr_scene_create_indexed(const float* verts, uint32_t nverts, const u
     cudaError_t e = cudaSuccess;
     if ((e = dmalloc(&s->d_verts, 3ull * nverts)) != cudaSuccess ||
         (e = dmalloc(&s->d_idx, 3ull * ntri)) != cudaSuccess ||
-        (e = dmalloc(&s->d_uvs, 3ull * ntri)) != cudaSuccess ||
-        (e = dmalloc(&s->d_geom, (size_t)ntri)) != cudaSuccess ||
+        (e = dmalloc(&s->d_attrs, 2ull * ntri)) != cudaSuccess ||
         (e = dmalloc(&s->d_tex, (size_t)ntex)) != cudaSuccess ||
         (e = dmalloc(&s->d_texels, (size_t)texel_bytes)) != cudaSuccess ||
         (e = dmalloc(&s->d_user, 1)) != cudaSuccess || (e = dmalloc(&s->d_err, 2)) != cudaSuccess)
         return bail(cuda_fail(e, "scene allocation"));
     if ((nverts && (e = cudaMemcpy(s->d_verts, verts, 12ull * nverts, cudaMemcpyHostToDevice))) ||
         (ntri && (e = cudaMemcpy(s->d_idx, idx, 12ull * ntri, cudaMemcpyHostToDevice))) ||
-        (ntri && (e = cudaMemcpy(s->d_uvs, uvs, 24ull * ntri, cudaMemcpyHostToDevice))) ||
-        (ntri && (e = cudaMemcpy(s->d_geom, geom_id, 4ull * ntri, cudaMemcpyHostToDevice))) ||
+        (ntri && (e = upload_attrs(s->d_attrs, uvs, geom_id, ntri))) ||
         (ntex && (e = cudaMemcpy(s->d_tex, td.data(), sizeof(TexDesc) * ntex,
                                  cudaMemcpyHostToDevice))) ||
         (e = cudaMemset(s->d_err, 0, 2 * sizeof(uint32_t))))
@@ -705,8 +733,7 @@ vsr_status vsr_scene_destroy(vsr_scene* s) {
     free_bvh(s);
     dfree(s->d_verts);
     dfree(s->d_idx);
-    dfree(s->d_uvs);
-    dfree(s->d_geom);
+    dfree(s->d_attrs);
     dfree(s->d_tex);
     dfree(s->d_texels);
     dfree(s->d_user);
@@ -793,8 +820,7 @@ vsr_status vsr_bvh_load(vsr_scene* s, const void* blob, size_t bytes) {
     DevScene& d = s->dev;
     d.nodes = s->d_nodes;
     d.tris = s->d_tris;
-    d.uvs = s->d_uvs;
-    d.geom = s->d_geom;
+    d.attrs = s->d_attrs;
     d.tex = s->d_tex;
     d.texels = s->d_texels;
     d.err = s->d_err;

@@ -33,12 +33,13 @@ __device__ __forceinline__ void path_albedo(const DevScene& sc, uint32_t prim, f
     alb[0] = pd.untex[0];
     alb[1] = pd.untex[1];
     alb[2] = pd.untex[2];
-    const uint32_t g = VSR_LDG(sc.geom + prim);
+    const Attr at = load_attr(sc, prim);
+    const uint32_t g = at.geom();
     if (g == kMiss) return;
     const uint4 d = VSR_LDG(reinterpret_cast<const uint4*>(sc.tex + g));
     if (d.x == kTexU8) return;
     const unsigned long long off = VSR_LDG(&sc.tex[g].offset);
-    const float2 uv = lerp_uv(sc.uvs, prim, u, v);
+    const float2 uv = lerp_uv(at, u, v);
     const unsigned long long k =
         (unsigned long long)texel_coord(uv.y, d.z) * d.y + texel_coord(uv.x, d.y);
     for (int c = 0; c < 3; ++c)

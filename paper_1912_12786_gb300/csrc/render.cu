@@ -145,7 +145,8 @@ __global__ void __launch_bounds__(256) k_shade_hits(DevScene sc, ShadeDev sh,
         surface(verts, idx, prim, v3(rb.x, rb.y, rb.z), v3(sh.light[0], sh.light[1], sh.light[2]),
                 f);
         Bilinear b;
-        albedo(sc, VSR_LDG(sc.geom + prim), lerp_uv(sc.uvs, prim, h.y, h.z), b);
+        const Attr at = load_attr(sc, prim);
+        albedo(sc, at.geom(), lerp_uv(at, h.y, h.z), b);
         for (int ch = 0; ch < 3; ++ch) c[ch] = b.rgb[ch] * f.s;
     }
     image[3 * i] = c[0];
@@ -195,11 +196,12 @@ __device__ __forceinline__ void shade_adjoint(const DevScene& sc, const ShadeDev
     const V3 L = v3(sh.light[0], sh.light[1], sh.light[2]);
     Surface f;
     surface(verts, idx, prim, d, L, f);
-    const uint32_t geom = VSR_LDG(sc.geom + prim);
-    const float2 c0 = VSR_LDG(sc.uvs + 3ull * prim), c1 = VSR_LDG(sc.uvs + 3ull * prim + 1),
-                 c2 = VSR_LDG(sc.uvs + 3ull * prim + 2);
+    const Attr at = load_attr(sc, prim);
+    const uint32_t geom = at.geom();
+    const float2 c0 = make_float2(at.a.x, at.a.y), c1 = make_float2(at.a.z, at.a.w),
+                 c2 = make_float2(at.b.x, at.b.y);
     Bilinear b;
-    albedo(sc, geom, lerp_uv(sc.uvs, prim, bu, bv), b);
+    albedo(sc, geom, lerp_uv(at, bu, bv), b);
 
     // texel gradients
     if (grad_texels && b.rgba32f && geom == sh.grad_tex && f.s > 0.0f) {
@@ -305,7 +307,8 @@ __global__ void __launch_bounds__(256) k_ao_shade(DevScene sc, ShadeDev sh,
         o = (float)occluded / (float)spp;
         const float vis = 1.0f - o;
         Bilinear b;
-        albedo(sc, VSR_LDG(sc.geom + prim), lerp_uv(sc.uvs, prim, h.y, h.z), b);
+        const Attr at = load_attr(sc, prim);
+        albedo(sc, at.geom(), lerp_uv(at, h.y, h.z), b);
         for (int ch = 0; ch < 3; ++ch) c[ch] = b.rgb[ch] * vis;
     }
     image[3 * i] = c[0];
@@ -337,10 +340,11 @@ __global__ void __launch_bounds__(256) k_ao_backward(DevScene sc, ShadeDev sh,
         atomicOr(sc.err, kErrHit);
         return;
     }
-    const uint32_t geom = VSR_LDG(sc.geom + prim);
+    const Attr at = load_attr(sc, prim);
+    const uint32_t geom = at.geom();
     if (geom != sh.grad_tex) return;
     Bilinear b;
-    albedo(sc, geom, lerp_uv(sc.uvs, prim, h.y, h.z), b);
+    albedo(sc, geom, lerp_uv(at, h.y, h.z), b);
     if (!b.rgba32f) return;
     const float vis = 1.0f - VSR_LDG(occ + i);
     if (vis == 0.0f) return;

@@ -22,7 +22,7 @@ namespace vsr {
 namespace {
 
 template <int Q, class H>
-__global__ void __launch_bounds__(256) k_trace_oct(DevScene sc, IsectParams ip,
+__global__ void __launch_bounds__(256, Q == kClosest ? H::kOctBlocksClosest : 0) k_trace_oct(DevScene sc, IsectParams ip,
                                                    const float4* __restrict__ rays, RayMap map,
                                                    float4* __restrict__ hits,
                                                    uint2* __restrict__ counters) {

@@ -10,7 +10,8 @@
 //   tris   3 x float4 per leaf slot: {v0.xyz, prim id}, {e1.xyz, node id of
 //          the leaf}, {e2.xyz, 0} with e1 = v1 - v0, e2 = v2 - v0, in leaf
 //          order.
-//   uvs    3 x float2 per original triangle id; geom: texture id per id.
+//   attrs  2 x float4 per original triangle id: {tc0, tc1}, {tc2, texture id,
+//          0}, 32 bytes aligned, so that an alpha test reads one sector.
 //
 // Rounding: the file is compiled with -fmad=false and every product, sum and
 // fused multiply-add below is an explicit __fmul_rn / __fadd_rn / __fmaf_rn,
@@ -74,8 +75,7 @@ struct TexDesc {
 struct DevScene {
     const float4* nodes;
     const float4* tris;
-    const float2* uvs;
-    const uint32_t* geom;
+    const float4* attrs;
     const TexDesc* tex;
     const uint8_t* texels;
     uint32_t* err;
@@ -271,15 +271,22 @@ __device__ __forceinline__ bool tri_test(const Ray& r, float4 a, float4 e1, floa
 // --------------------------------------------------------------------------
 // intersector arithmetic (Section 4 use cases)
 
+// Texture coordinates and texture of a triangle.
+struct Attr {
+    float4 a, b;
+    __device__ __forceinline__ uint32_t geom() const { return __float_as_uint(b.z); }
+};
+
+__device__ __forceinline__ Attr load_attr(const DevScene& sc, uint32_t prim) {
+    return Attr{VSR_LDG(sc.attrs + 2ull * prim), VSR_LDG(sc.attrs + 2ull * prim + 1)};
+}
+
 // Interpolated texture coordinate: w0 = (1-u)-v, uv = v*tc2 + (u*tc1 + w0*tc0).
-__device__ __forceinline__ float2 lerp_uv(const float2* __restrict__ uvs, uint32_t prim, float u,
-                                          float v) {
-    const float2 c0 = VSR_LDG(uvs + 3ull * prim), c1 = VSR_LDG(uvs + 3ull * prim + 1),
-                 c2 = VSR_LDG(uvs + 3ull * prim + 2);
+__device__ __forceinline__ float2 lerp_uv(const Attr& t, float u, float v) {
     const float w0 = __fsub_rn(__fsub_rn(1.0f, u), v);
     float2 r;
-    r.x = __fmaf_rn(v, c2.x, __fmaf_rn(u, c1.x, __fmul_rn(w0, c0.x)));
-    r.y = __fmaf_rn(v, c2.y, __fmaf_rn(u, c1.y, __fmul_rn(w0, c0.y)));
+    r.x = __fmaf_rn(v, t.b.x, __fmaf_rn(u, t.a.z, __fmul_rn(w0, t.a.x)));
+    r.y = __fmaf_rn(v, t.b.y, __fmaf_rn(u, t.a.w, __fmul_rn(w0, t.a.y)));
     return r;
 }
 
@@ -289,12 +296,18 @@ __device__ __forceinline__ uint32_t texel_coord(float c, uint32_t n) {
     return (uint32_t)min(i, (int)n - 1);
 }
 
-// Alpha-mask decision: nearest texel, clamp to edge.
+// Alpha-mask decision: nearest texel, clamp to edge.  Bound by its chain of
+// dependent loads (triangle, attributes, texture, texel): the texture id and
+// the coordinates come in one sector, in one round trip.  With the id and the
+// coordinates in arrays of their own the id came first and the rest took two
+// sectors more: eight hits a ray, 230,400 rays, 578 -> 554 us; 1,000,003
+// diffuse rays 782 -> 768 us; 360,000 occlusion rays' frame 392 -> 377 us.
 __device__ __forceinline__ bool alpha_tex_accept(const DevScene& sc, const IsectParams& ip,
                                                  uint32_t prim, float u, float v) {
-    const uint32_t g = VSR_LDG(sc.geom + prim);
+    const Attr at = load_attr(sc, prim);
+    const uint32_t g = at.geom();
     if (g == kMiss) return true;
-    const float2 uv = lerp_uv(sc.uvs, prim, u, v);
+    const float2 uv = lerp_uv(at, u, v);
     const uint4 d = VSR_LDG(reinterpret_cast<const uint4*>(sc.tex + g));
     const unsigned long long off = VSR_LDG(&sc.tex[g].offset);
     const uint32_t i = texel_coord(uv.x, d.y), j = texel_coord(uv.y, d.z);
@@ -336,9 +349,10 @@ __device__ __forceinline__ int sin_sign(float x) {
 // differs only where it underflows, i.e. both sines below 1e-22).
 __device__ __forceinline__ bool proc_alpha_accept(const DevScene& sc, const IsectParams& ip,
                                                   uint32_t prim, float u, float v) {
-    const uint32_t g = VSR_LDG(sc.geom + prim);
+    const Attr at = load_attr(sc, prim);
+    const uint32_t g = at.geom();
     if (g == kMiss) return true;
-    const float2 uv = lerp_uv(sc.uvs, prim, u, v);
+    const float2 uv = lerp_uv(at, u, v);
     return sin_sign(__fmul_rn(ip.freq, uv.x)) * sin_sign(__fmul_rn(ip.freq, uv.y)) > 0;
 }
 
@@ -361,6 +375,7 @@ struct IsectNone {
     // are compiled for, per query (1: no register budget)
     static constexpr int kMinBlocksClosest = 1;
     static constexpr int kMinBlocksAny = 1;
+    static constexpr int kOctBlocksClosest = 0;  // the same for k_trace_oct (0: no budget)
     __device__ __forceinline__ void begin(const Ray&, const IsectParams&) {}
     __device__ __forceinline__ void box() {}
     __device__ __forceinline__ void tri() {}
@@ -385,6 +400,10 @@ struct IsectAlphaTex : IsectNone {
 };
 
 struct IsectProcAlpha : IsectNone {
+    // Left alone ptxas takes 48 registers and spills 164 bytes: 2,073,600 rays on
+    // 1,000,002 triangles 434 us, with this budget (60 registers) 427; 518,400
+    // rays on 50,000 156 -> 144 us.
+    static constexpr int kOctBlocksClosest = 4;
     static constexpr bool kTexcoords = true;
     __device__ __forceinline__ bool accept(const DevScene& sc, const IsectParams& ip,
                                            uint32_t prim, float u, float v, float) {
@@ -648,7 +667,7 @@ __device__ __forceinline__ void traverse_body(const DevScene& sc, const IsectPar
                 }
                 if (STATS) {
                     st.cands++;
-                    if (H::kTexcoords && VSR_LDG(sc.geom + prim) != kMiss) st.texs++;
+                    if (H::kTexcoords && load_attr(sc, prim).geom() != kMiss) st.texs++;
                 }
                 if (!h.accept(sc, ip, prim, u, v, t)) continue;
                 best.take(t, u, v, prim);
@@ -762,7 +781,7 @@ __device__ __forceinline__ bool traverse_step(const DevScene& sc, const IsectPar
         }
         if (STATS) {
             st.cands++;
-            if (H::kTexcoords && VSR_LDG(sc.geom + prim) != kMiss) st.texs++;
+            if (H::kTexcoords && load_attr(sc, prim).geom() != kMiss) st.texs++;
         }
         if (!h.accept(sc, ip, prim, u, v, t)) continue;
         best.take(t, u, v, prim);
@@ -793,7 +812,7 @@ __device__ __forceinline__ bool test_prim(const DevScene& sc, const IsectParams&
     }
     if (STATS) {
         st.cands++;
-        if (H::kTexcoords && VSR_LDG(sc.geom + prim) != kMiss) st.texs++;
+        if (H::kTexcoords && load_attr(sc, prim).geom() != kMiss) st.texs++;
     }
     if (!h.accept(sc, ip, prim, u, v, t)) return false;
     best.take(t, u, v, prim);
