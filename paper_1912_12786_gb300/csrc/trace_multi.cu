@@ -8,7 +8,7 @@
 // candidates that would enter the buffer; with n == 1 it is the closest-hit
 // query.  The intersector is compiled in (static dispatch) or reached
 // through this module's callback tables (dynamic dispatch, dynamic.cuh).
-// Launch shapes: one ray per thread, or persistent warps with per-lane loops
+// Launch shapes: one ray per thread, or persistent warps, each with per-lane loops
 // or in lock step.
 //
 // The first launch of the unchecked build raised a misaligned-address fault
@@ -18,6 +18,8 @@
 // path and the hit and counter stores check their address: a misaligned
 // access is skipped and its source line reported (device error bit 2).
 #define VSR_CHECKED_LOADS 1
+#include <type_traits>
+
 #include "dynamic.cuh"
 
 namespace vsr {
@@ -98,6 +100,47 @@ __global__ void __launch_bounds__(256) k_trace_multi(DevScene sc, IsectParams ip
     stk.init(s_stack + threadIdx.x, stride);
     traverse_body<kClosest, H, false>(sc, ip, r, h, mb, st, stk);
     write_multi(r, verts, idx, mb, h, i, nh, hits, counters);
+}
+
+// One ray per thread, the warp in lock step (warp_step; every lane stays in the
+// loop to the end, since each pass ends in a full-warp vote).  Rays that go on
+// past their first hits drift apart: the per-lane loops kept 14.4 of 32 lanes
+// busy on eight hits a ray, and both forms are bound by the latency of the node
+// and triangle loads at 32 resident warps.  230,400 camera rays on a forest of
+// 200,002 triangles, eight hits: 524 -> 452 us; 400,000 on 100,000 quads, 16
+// hits: 432 -> 317; one hit: equal (234 -> 230).  The budget keeps the alpha
+// mask at 64 registers (74 otherwise: 479).
+template <class H>
+__global__ void __launch_bounds__(256, 4) k_trace_multi_ls(
+    DevScene sc, IsectParams ip, const float* __restrict__ verts,
+    const uint32_t* __restrict__ idx, const float4* __restrict__ rays, RayMap map, uint32_t nh,
+    float4* __restrict__ hits, uint2* __restrict__ counters) {
+    extern __shared__ uint32_t s_stack[];
+    const unsigned long long g = slot_of_thread(map);
+    const unsigned long long i = g < map.threads ? ray_of_thread(g, map) : map.n;
+    const bool live = i < map.n;
+    const uint32_t stride = blockDim.x;
+    uint32_t* buf = s_stack + sc.stack_depth * stride;
+    MultiBest mb;
+    mb.tk = reinterpret_cast<float*>(buf) + threadIdx.x;
+    mb.pk = buf + nh * stride + threadIdx.x;
+    mb.stride = stride;
+    mb.n = nh;
+    ShortStack<0> stk;
+    stk.init(s_stack + threadIdx.x, stride);
+    Ray r{};
+    Stats st;
+    H h;
+    uint32_t ref = 0, steps = 0;
+    bool busy = false;
+    if (live) {
+        r = make_ray(VSR_LDG(rays + 2 * i), VSR_LDG(rays + 2 * i + 1));
+        busy = traverse_start<kClosest, H, false>(sc, ip, r, h, mb, st, ref, steps, stk);
+    }
+    while (__any_sync(kFullMask, busy))
+        if (warp_step<kClosest, H, false>(sc, ip, r, h, mb, st, busy, ref, steps, stk))
+            busy = false;
+    if (live) write_multi(r, verts, idx, mb, h, i, nh, hits, counters);
 }
 
 // Persistent multi-hit (persistent_rays: warps claim rays from a counter and
@@ -196,17 +239,24 @@ cudaError_t multi_one(const LaunchArgs& a, const float* verts, const uint32_t* i
         return a.lockstep ? multi_persistent<H, true>(a, verts, idx, nh)
                           : multi_persistent<H, false>(a, verts, idx, nh);
     const size_t smem = ((size_t)a.sc.stack_depth + 2u * nh) * a.block * sizeof(uint32_t);
-    auto k = k_trace_multi<H>;
-    if (smem > 48 * 1024) {
-        cudaError_t e =
-            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
     RayMap map = a.map;
     const unsigned long long grid = (spread_rays(map, kSpreadWarps) + a.block - 1) / a.block;
-    k<<<(unsigned)grid, a.block, smem, a.stream>>>(a.sc, a.ip, verts, idx, a.rays, map, nh,
-                                                     a.hits, a.counters, a.dyn_user);
-    return cudaGetLastError();
+    auto go = [&](auto k, auto... more) {
+        if (smem > 48 * 1024) {
+            cudaError_t e =
+                cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        k<<<(unsigned)grid, a.block, smem, a.stream>>>(a.sc, a.ip, verts, idx, a.rays, map, nh,
+                                                       a.hits, a.counters, more...);
+        return cudaGetLastError();
+    };
+    // Warps with fewer than eight rays have little to share, and the votes cost
+    // them more than they bring: 10,000 rays 77 us per lane and 85 in lock step,
+    // 18,000 rays 108 and 105, 22,400 rays (eight a warp) 141 and 126.
+    if constexpr (!std::is_same<H, IsectDynamic>::value)
+        if (map.lane_bits >= 3) return go(k_trace_multi_ls<H>);
+    return go(k_trace_multi<H>, a.dyn_user);
 }
 
 }  // namespace
