@@ -537,8 +537,9 @@ cudaError_t time_params(const LaunchArgs& base, const vsr_trace_params& c, int k
 // candidates on the caller's rays, and remember it in the scene.  First pass:
 // one ray per thread, per-lane loops and lock step x block 64/128/256 x
 // register-stack depth 0/1/2/4/8 (static dispatch; dynamic: depth 0),
-// starting from the default (128, 0, per-lane loops); then the best of these
-// in coherence order (its sort timed with it); last, the persistent launch at
+// starting from the default (128, 0, per-lane loops), and for any hit in buffer
+// order the octant-specialised box test; then the best of these in coherence
+// order (its sort timed with it); last, the persistent launch at
 // the best configuration with per-lane loops and in lock step, refill
 // thresholds 1/8/16/24.  Every candidate but the coherence-order one keeps
 // the caller's image_width.
@@ -574,6 +575,13 @@ vsr_status tune_trace(vsr_scene* s, const LaunchArgs& base, const vsr_intersecto
             for (uint32_t k : {0u, 1u, 2u, 4u, 8u})
                 if ((!dynamic || k == 0) && !(b == 128u && k == 0u && ls == 0u))
                     consider(vsr_trace_params{b, 0u, 16u, 0u, image_width, k, 0u, 0u, 0u, 0u, ls});
+    if (!dynamic && query == kAny && image_width == 0)
+        // elsewhere the octant-dispatching kernel runs with octant 0 too
+        for (uint32_t b : {64u, 128u, 256u}) {
+            vsr_trace_params c{b, 0u, 16u, 0u, image_width, 0u, 0u, 0u, 0u, 0u, 0u};
+            c.octant = 1u;
+            consider(c);
+        }
     if (base.n <= coherence_sort_max_rays()) {
         // the fastest one-ray-per-thread configuration in coherence order
         // (the sort is part of every timed launch)
@@ -590,6 +598,7 @@ vsr_status tune_trace(vsr_scene* s, const LaunchArgs& base, const vsr_intersecto
                 c.persistent = 1u;
                 c.refill_threshold = r;
                 c.lockstep = ls;
+                c.octant = 0u;
                 if (ls) c.stack_regs = 0u;  // the two-level records take no others
                 consider(c);
             }

@@ -11,18 +11,32 @@
 // test the same boxes with the same outcome, so the nodes, leaves, hits and
 // counts are those of k_trace bit for bit.
 //
-// These kernels run every static launch of that shape, asked for (octant 1) or
-// not: the vote costs rays that point anywhere nothing that shows (diffuse
-// rays 1,383 us against 1,393 with the generic kernel alone), and camera rays
-// gain (forest frame 524 -> 475 us, heat map of 1283 x 719 154 -> 133 us).
+// Which launches of that shape run these kernels without asking for it (octant
+// 1): launch_static.  Camera rays gain (forest frame 524 -> 475 us, heat map of
+// 1283 x 719 154 -> 133 us), and the vote costs mixed warps nothing that shows.
 #include "trace_static.cuh"
 
 namespace vsr {
 
 namespace {
 
+// Resident warps the kernel is compiled for: 36 per SM (56 registers), and 40 (48
+// registers, 20 bytes spilled) for the any-hit alpha masks, which wait on more
+// loads.  Left alone ptxas takes 58 to 62 registers for most kinds, 32 warps, and
+// 48 with 164 bytes of spills for the closest procedural hit.  1,000,003 diffuse
+// rays, us without / with: closest default 1,056 / 985, procedural 1,466 / 1,399,
+// count 1,043 / 998, any count 1,004 / 945; 2,073,600 camera rays in rows on the
+// forest: default 378 / 371, procedural 602 / 586, any count 140 / 134.  The masks'
+// any hit at 36 warps instead of 40: 1,342 / 1,397.
 template <int Q, class H>
-__global__ void __launch_bounds__(256, Q == kClosest ? H::kOctBlocksClosest : 0) k_trace_oct(DevScene sc, IsectParams ip,
+struct OctBudget {
+    static constexpr bool kMask = Q == kAny && H::kTexcoords;
+    static constexpr int kThreads = kMask ? 256 : 384, kBlocks = kMask ? 5 : 3;
+};
+
+template <int Q, class H>
+__global__ void __launch_bounds__(OctBudget<Q, H>::kThreads, OctBudget<Q, H>::kBlocks)
+                                       k_trace_oct(DevScene sc, IsectParams ip,
                                                    const float4* __restrict__ rays, RayMap map,
                                                    float4* __restrict__ hits,
                                                    uint2* __restrict__ counters) {

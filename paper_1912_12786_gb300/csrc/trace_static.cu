@@ -27,9 +27,15 @@ cudaError_t launch_static(const LaunchArgs& a, int kind, bool stats) {
         b.lockstep = 1u;
         if (walks_records(b, kind)) return launch_wide(b, kind);
     }
-    // the octant-dispatching kernel also runs the launches that do not ask for
-    // it (trace_oct.cu)
-    if (a.octant || (!a.persistent && !a.lockstep && a.stack_regs == 0))
+    // The octant-dispatching kernel also runs launches that do not ask for it: on
+    // pixel tiles, with few rays, which it spreads, and every closest hit (mixed
+    // warps are no slower in it: 1,000,003 diffuse rays, default 985 us against
+    // 1,038, alpha mask 1,396 / 1,398; camera rays in rows gain 4 to 18%).  Any hit
+    // in buffer order keeps the generic kernel, where rays that point anywhere are
+    // 1 to 3% faster (default 927 / 955, alpha mask 1,322 / 1,344).
+    if (a.octant || (!a.persistent && !a.lockstep && a.stack_regs == 0 &&
+                     (a.query == kClosest || a.map.width > 0 ||
+                      spreads_rays(a.map, kSpreadWarps))))
         return launch_static_octant(a, kind);
     switch (a.stack_regs) {
         case 0: return launch_static_k0(a, kind, false);

@@ -257,8 +257,6 @@ cudaError_t launch_shape(const LaunchArgs& a) {
     if (a.persistent) return launch_persistent<Q, H, STATS, K, LS>(a);
     if constexpr (LS) {
         return launch_lockstep<Q, H, STATS, K>(a);
-    } else if constexpr (K == 0 && !STATS) {
-        return cudaErrorInvalidValue;  // k_trace_oct's launches
     } else {
         const size_t smem = (size_t)stack_words(a.sc.stack_depth, K) * a.block * sizeof(uint32_t);
         const unsigned long long grid = (a.map.threads + a.block - 1) / a.block;

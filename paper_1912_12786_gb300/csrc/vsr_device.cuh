@@ -375,7 +375,6 @@ struct IsectNone {
     // are compiled for, per query (1: no register budget)
     static constexpr int kMinBlocksClosest = 1;
     static constexpr int kMinBlocksAny = 1;
-    static constexpr int kOctBlocksClosest = 0;  // the same for k_trace_oct (0: no budget)
     __device__ __forceinline__ void begin(const Ray&, const IsectParams&) {}
     __device__ __forceinline__ void box() {}
     __device__ __forceinline__ void tri() {}
@@ -400,10 +399,6 @@ struct IsectAlphaTex : IsectNone {
 };
 
 struct IsectProcAlpha : IsectNone {
-    // Left alone ptxas takes 48 registers and spills 164 bytes: 2,073,600 rays on
-    // 1,000,002 triangles 434 us, with this budget (60 registers) 427; 518,400
-    // rays on 50,000 156 -> 144 us.
-    static constexpr int kOctBlocksClosest = 4;
     static constexpr bool kTexcoords = true;
     __device__ __forceinline__ bool accept(const DevScene& sc, const IsectParams& ip,
                                            uint32_t prim, float u, float v, float) {

@@ -103,6 +103,10 @@ inline unsigned long long spread_rays(RayMap& map, unsigned warps_per_sm) {
     while (map.lane_bits > 0 && (map.threads >> (map.lane_bits - 1)) <= warps) --map.lane_bits;
     return ((map.threads + (1ull << map.lane_bits) - 1) >> map.lane_bits) * 32ull;
 }
+inline bool spreads_rays(RayMap map, unsigned warps_per_sm) {
+    spread_rays(map, warps_per_sm);
+    return map.lane_bits < 5u;
+}
 
 // Stream-ordered scratch (scratch.cu), freed with cudaFreeAsync.  The pool lives
 // while scenes do; both notes are for the current device.
