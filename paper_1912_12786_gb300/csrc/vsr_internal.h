@@ -94,10 +94,23 @@ inline int persistent_grid(const LaunchArgs& a, const void* kernel, size_t smem)
 // Random quads would take more warps, but neighbouring camera rays that agree
 // (the forest) lose once the warps no longer fit the chip at once: the line is
 // what stays resident, 36 warps of the octant kernels' 56 registers, 24 of the
-// kernels with 78 to 80.  Sets map.lane_bits; returns the launch's threads.
-constexpr unsigned kSpreadWarps = 36, kSpreadWarpsLarge = 24;
+// kernels with 78 to 80.  In buffer order a warp's rays share less and every
+// further warp loads nodes of its own, from DRAM when the caches are cold (the
+// table above is warm), so there the line is 14 for all kernels: camera rays
+// through random pixels, forest of 200,002 triangles, L2 flushed, us with lines
+// of 0 / 9 / 18 / 36 warps per SM:
+//   rays     default, closest hit     alpha texture, any hit
+//   4,000    64 / 44 / 42 / 38        72 / 58 / 56 / 52
+//   20,000   66 / 64 / 62 / 72        81 / 68 / 66 / 58
+//   40,000   70 / 70 / 72 / 91        78 / 78 / 66 / 66
+//   80,000   85 / 85 / 85 / 109       78 / 78 / 78 / 76
+// (1,000,002 triangles, 40,000 rays, default closest hit: 81 / 81 / 89 / 103);
+// pixel tiles at 51,200 rays 44 / 44 / 44 / 44 there and 85 / 83 / 83 / 64 on
+// 5,000 quads.  Sets map.lane_bits; returns the launch's threads.
+constexpr unsigned kSpreadWarps = 36, kSpreadWarpsLarge = 24, kSpreadWarpsRows = 14;
 int sm_count();  // of the current device
 inline unsigned long long spread_rays(RayMap& map, unsigned warps_per_sm) {
+    if (map.width == 0 && warps_per_sm > kSpreadWarpsRows) warps_per_sm = kSpreadWarpsRows;
     const unsigned long long warps = (unsigned long long)warps_per_sm * (unsigned)sm_count();
     map.lane_bits = 5;
     while (map.lane_bits > 0 && (map.threads >> (map.lane_bits - 1)) <= warps) --map.lane_bits;

@@ -41,9 +41,10 @@ def _rays(sc, n):
     return r.float().contiguous().cuda()
 
 
-def line(V):
-    """Rays from which on a warp of the one-ray-per-thread launch takes eight."""
-    return 36 * torch.cuda.get_device_properties(0).multi_processor_count * 4
+def line(warps):
+    """Rays from which on a warp of the one-ray-per-thread launch takes eight,
+    spread over `warps` warps per SM (14 in buffer order, 36 on pixel tiles)."""
+    return warps * torch.cuda.get_device_properties(0).multi_processor_count * 4
 
 
 @pytest.mark.parametrize("kind", ["none", "default", "alpha_tex", "proc_alpha", "count"])
@@ -51,9 +52,9 @@ def line(V):
 def test_lockstep_equals_per_lane(V, scene, kind, nh):
     sc, s = scene
     i = V.intersector(kind)
-    n0 = line(V)
-    for n, width in ((1, 0), (33, 0), (n0, 0), (n0 + 1, 0), (n0 + 31, 0), (301 * 203, 301),
-                     (301 * 203 - 5, 301)):
+    n0, n1 = line(14), line(36)
+    for n, width in ((1, 0), (33, 0), (n0, 0), (n0 + 1, 0), (n0 + 31, 0), (n1, 64),
+                     (n1 + 1, 64), (301 * 203, 301), (301 * 203 - 5, 301)):
         rays = _rays(sc, n)
         out = []
         for persistent in (0, 1):
