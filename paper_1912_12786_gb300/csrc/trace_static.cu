@@ -22,10 +22,11 @@ cudaError_t launch_static(const LaunchArgs& a, int kind, bool stats) {
     if (a.reg_cap >= 3) return launch_static_capped(a, kind, a.reg_cap);
     if (walks_records(a, kind)) return launch_wide(a, kind);
     // a shape that leaves the traversal's form open (records_limit, api.cu)
-    if (!a.persistent && !a.lockstep && !a.octant && a.reg_cap == 0 && a.n <= a.records_up_to) {
+    if (!a.persistent && !a.lockstep && !a.octant && a.reg_cap == 0 && a.stack_regs == 0 &&
+        kind <= 3 && a.n <= a.records_up_to) {
         LaunchArgs b = a;
         b.lockstep = 1u;
-        if (walks_records(b, kind)) return launch_wide(b, kind);
+        return walks_records(b, kind) ? launch_wide(b, kind) : launch_static_k0(b, kind, false);
     }
     // The octant-dispatching kernel also runs launches that do not ask for it: on
     // pixel tiles, with few rays, which it spreads, and every closest hit (mixed

@@ -243,11 +243,12 @@ cudaError_t launch_persistent(const LaunchArgs& a) {
 template <int Q, class H, bool STATS, int K, int MINB = min_blocks<Q, H>()>
 cudaError_t launch_lockstep(const LaunchArgs& a) {
     const size_t smem = (size_t)stack_words(a.sc.stack_depth, K) * a.block * sizeof(uint32_t);
-    const unsigned long long grid = (a.map.threads + a.block - 1) / a.block;
+    RayMap map = a.map;
+    const unsigned long long grid = (spread_rays(map, kSpreadWarpsLarge) + a.block - 1) / a.block;
     auto k = lockstep_kernel<Q, H, STATS, K, MINB>();
     cudaError_t e = ensure_smem(k, smem);
     if (e != cudaSuccess) return e;
-    k<<<(unsigned)grid, a.block, smem, a.stream>>>(a.sc, a.ip, a.rays, a.map, a.hits, a.counters,
+    k<<<(unsigned)grid, a.block, smem, a.stream>>>(a.sc, a.ip, a.rays, map, a.hits, a.counters,
                                                      a.stats, a.dyn_user);
     return cudaGetLastError();
 }

@@ -89,8 +89,18 @@ cudaError_t wide_kind(const LaunchArgs& a, int kind) {
 
 }  // namespace
 
+// Lock step walks the records on trees with long descents (records_limit), for
+// rays in buffer order; on other trees, whose nodes stay in L1, and on pixel tiles
+// a record costs more instructions than it saves round trips.  Persistent, L2
+// flushed, alpha texture, us records / binary nodes:
+//   500,000 diffuse rays, closest and any hit: quads 1,000 141/131 129/129, 5,000
+//   301/283 272/267, 50,000 391/394 365/380, 500,000 579/593 546/582; occlusion
+//   rays on 50,000 134/144 127/142; forest 200,002 1,622/1,421 463/449
+//   400,000 camera rays on tiles: quads 50,000 169/166 164/156, 400,000 264/251
+//   249/241; forest 1,000,002 at 1080p 866/684 551/474
 bool walks_records(const LaunchArgs& a, int kind) {
-    return a.sc.wide && !a.binary_nodes && kind >= 0 && kind <= 3 && a.lockstep && a.stack_regs == 0;
+    return a.sc.wide && a.records_up_to > 0 && a.map.width == 0 && !a.binary_nodes &&
+           kind >= 0 && kind <= 3 && a.lockstep && a.stack_regs == 0;
 }
 
 cudaError_t launch_wide(const LaunchArgs& a, int kind) {

@@ -88,12 +88,19 @@ def _rays(sc, n=6000, seed=3):
 
 def _same(V, s, d, kind, query, label):
     n = d.shape[0]
-    out = [torch.full((n, 4), 7.0, device="cuda") for _ in range(3)]
+    out = [torch.full((n, 4), 7.0, device="cuda") for _ in range(4)]
     isect = V.intersector(kind)
     V.vsr_trace(s, d, isect, query, out[0], None, V.trace_params(block_size=64))
     V.vsr_trace(s, d, isect, query, out[1], None, V.trace_params(block_size=96, lockstep=1))
     V.vsr_trace(s, d, isect, query, out[2], None,
                 V.trace_params(block_size=64, lockstep=1, persistent=1, refill_threshold=24))
+    # a batch walks the records of any tree; the launches above those of trees
+    # with long descents
+    b = V.vsr_batch_create([s], [d], [out[3]], isect, query,
+                           V.trace_params(block_size=64, lockstep=1))
+    V.vsr_batch_launch(b)
+    torch.cuda.synchronize()
+    V.vsr_batch_destroy(b)
     assert V.vsr_get_device_error(s) == 0, label
     want = out[0].view(torch.int32)
     for k, h in enumerate(out[1:]):
@@ -163,5 +170,6 @@ def test_open_launches_match_binary(V, n_quads, n):
             V.vsr_trace_stats(s, d, V.intersector(kind), query, want, stats)
             V.vsr_trace(s, d, V.intersector(kind), query, got, None, V.trace_params())
             assert torch.equal(got.view(torch.int32), want.view(torch.int32)), (kind, query)
+            _same(V, s, d, kind, query, f"{n_quads}/{kind}/{query}")
     assert V.vsr_get_device_error(s) == 0
     s.close()
