@@ -68,9 +68,8 @@ def default_params(V, image_width=FRAME_W):
 
 
 def octant_params(V, image_width=FRAME_W):
-    """One ray per thread on 4x8 pixel tiles, block 64, with the box test
-    specialised to a warp's direction octant (static dispatch; what the
-    tuner picks on the forest frame)."""
+    """One ray per thread on 4x8 pixel tiles, block 64 (static dispatch; the
+    kernel specialises the box test to a warp's direction octant)."""
     p = default_params(V, image_width)
     p.block_size = 64
     p.octant = 1
@@ -78,10 +77,11 @@ def octant_params(V, image_width=FRAME_W):
 
 
 # the device code of the static trace kernels (the dominant kernel): the
-# kernel templates and the traversal they inline, and the octant-dispatching
-# kernel (vsr_internal.h adds host-side launch structures only; trace_k<K>.cu
+# kernel templates and the traversal they inline, the octant-dispatching
+# kernel and the walk over the two-level records (vsr_internal.h adds host-side launch structures only; trace_k<K>.cu
 # only instantiate)
-TRACE_SOURCES = ("trace_static.cuh", "vsr_device.cuh", "trace_oct.cu")
+TRACE_SOURCES = ("trace_static.cuh", "vsr_device.cuh", "trace_oct.cu", "wide.cuh",
+                 "trace_wide.cu")
 
 
 def kernel_source_hash() -> str:
@@ -974,30 +974,6 @@ def breakdown(V, s, d_rays, rays_s, n, flush, stream, torch, reps=5):
                     if r >= 2:
                         ms.append(e0.elapsed_time(e1))
                 res[f"stack_regs/{q}/block{block}/K{k}_ms"] = round(statistics.median(ms), 4)
-    # box tests specialised to the direction octant a warp's rays share,
-    # against the generic test: every static intersector, both passes, same
-    # tiles, launches interleaved
-    for kind in ("default", "alpha_tex", "proc_alpha", "count"):
-        isect = V.intersector(kind)
-        c = cnt if kind == "count" else None
-        for q, rr in (("closest", d_rays), ("any", rays_s)):
-            ms = {0: [], 1: []}
-            for r in range(reps + 2):
-                for oc in (0, 1):
-                    p = V.trace_params(block_size=128, image_width=FRAME_W, octant=oc)
-                    flush.zero_()
-                    e0 = torch.cuda.Event(enable_timing=True)
-                    e1 = torch.cuda.Event(enable_timing=True)
-                    e0.record(stream)
-                    V.vsr_trace(s, rr, isect, q, hits, c, p, stream)
-                    e1.record(stream)
-                    e1.synchronize()
-                    if r >= 2:
-                        ms[oc].append(e0.elapsed_time(e1))
-            t0, t1 = statistics.median(ms[0]), statistics.median(ms[1])
-            res[f"octant/{q}/{kind}/generic_ms"] = round(t0, 4)
-            res[f"octant/{q}/{kind}/octant_ms"] = round(t1, 4)
-            res[f"octant/{q}/{kind}/speedup"] = round(t0 / t1, 4)
     return res
 
 
@@ -1053,7 +1029,7 @@ def multi_hit(V, s, d_rays, n, flush, stream, torch, reps=5):
 def path_bench(V, s, sc, d_rays, n, flush, stream, torch, steps, bounces=3):
     """Diffuse path tracing of the forest frame: every segment a closest-hit
     query with the alpha intersector (primary segments on pixel tiles, bounce
-    segments over the live paths compacted after each bounce), 3 bounces,
+    segments over the list of the paths that go on), 3 bounces,
     sky light."""
     from paper_1912_12786_gb300.inputs import scenes
     dirs = torch.from_numpy(scenes.path_dirs(n, bounces)).to(d_rays.device)

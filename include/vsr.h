@@ -244,8 +244,8 @@ typedef struct vsr_trace_params {
                                   (persistent 0, lockstep 0), stack_regs 0,
                                   reg_cap_blocks 0 or 1; vsr_trace,
                                   vsr_render and vsr_path_trace; other entry
-                                  points take 0.  Launches of this shape do
-                                  so with 0 too. */
+                                  points take 0.  With 0 the library decides
+                                  for launches of this shape. */
 } vsr_trace_params;
 
 typedef struct vsr_scene vsr_scene;

@@ -297,7 +297,8 @@ void free_bvh(vsr_scene* s) {
 }
 
 // Up to how many rays a static launch of one ray per thread that leaves the
-// traversal's form open runs in lock step over the records.  That pays where a
+// traversal's form open runs in lock step (walks_records: over the records in
+// buffer order); 0 also keeps every launch off the records.  That pays where a
 // ray descends through many boxes per leaf, because lanes then reach their
 // leaves far apart even when neighbouring rays agree; the surface areas of the
 // boxes tell, relative to the root's the expected visits of a ray that crosses
