@@ -586,9 +586,10 @@ def run_ours(args):
     # Launch configuration: vsr_trace_tune times its candidates on the frame
     # (untimed, before the steps) and keeps the fastest in the scene for each
     # query; the timed step then calls vsr_trace with params NULL.  With
-    # --launch octant the step passes the configuration the tuner picks on
-    # this frame explicitly and nothing is tuned (for profiler runs, whose
-    # serialised launches would distort the tuner's timings).
+    # --launch octant the step passes block 64, one ray per thread, explicitly
+    # (within 1% of what the tuner picks on this frame) and nothing is tuned
+    # (for profiler runs, whose serialised launches would distort the tuner's
+    # timings).
     if args.launch == "octant":
         tuned_p = tuned_s = step_p = octant_params(V)
     else:
@@ -1540,8 +1541,7 @@ def main():
                     help="--leg trace/ao/batch_profile: 1 runs each warp in lock step")
     ap.add_argument("--launch", choices=["tuned", "octant"], default="tuned",
                     help="timed step: tuned = vsr_trace_tune first, then params NULL; octant = "
-                         "the configuration the tuner picks on the frame (block 64, pixel "
-                         "tiles, octant box test), passed explicitly, nothing tuned")
+                         "block 64 on pixel tiles passed explicitly, nothing tuned")
     ap.add_argument("--octant", type=int, default=0,
                     help="--leg trace/ao: 1 gives warps whose rays share a direction octant "
                          "a box test compiled for it")
