@@ -488,6 +488,9 @@ void bounce_launch(LaunchArgs& a) {
         a.block = 64u;
         a.refill = 24u;
         a.blocks_per_sm = 0u;
+        // the caller's watchdog is for persistent launches and none was asked
+        // for: a path it stopped would be shaded with an earlier segment's hit
+        a.wd = Watchdog{};
     }
 }
 
