@@ -399,8 +399,9 @@ vsr_status vsr_trace_multi(vsr_scene* scene, const vsr_ray* rays, uint64_t n,
  * `stream`.  The shading launch also lists the paths that go on (their order
  * may vary from run to run; results do not depend on it), and the next
  * segment's threads take the paths of that list.  Scratch (n * 68 bytes; 16
- * without bounces) comes from the stream-ordered allocator.  Errors as
- * vsr_trace.
+ * without bounces) comes from the stream-ordered allocator.  Where the
+ * watchdog of a persistent launch runs out (VSR_DEVERR_TIMEOUT), the radiance
+ * of paths it had not traced is undefined.  Errors as vsr_trace.
  */
 typedef struct vsr_path_params {
     uint32_t bounces;      /* 0..64 */
@@ -759,8 +760,9 @@ const char* vsr_last_error(void);
  *          count leaves);
  *   bit 2: a render or backward kernel found a load whose address did not
  *          match its width and skipped it (vsr_last_error() names the line);
- *   bit 3: a caller-supplied hit record named a primitive out of range
- *          (skipped; vsr_make_ao_rays gives its rays inactive);
+ *   bit 3: a hit record -- caller-supplied, or left over where the watchdog of
+ *          a render's or path's own trace ran out -- named a primitive out of
+ *          range (skipped; vsr_make_ao_rays gives its rays inactive);
  *   bit 4 (VSR_DEVERR_TIMEOUT): a persistent or batched launch ran out of
  *          its watchdog budget (vsr_trace_params.watchdog_iterations,
  *          watchdog_ms); the launch's results are incomplete.  A batch

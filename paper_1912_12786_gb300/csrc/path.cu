@@ -66,7 +66,11 @@ __device__ __forceinline__ bool shade_segment(
     const float4 h = VSR_LDG(hits + i);
     const uint32_t prim = __float_as_uint(h.w);
     bool done = false;
-    if (prim == kMiss) {
+    if (prim != kMiss && prim >= sc.nprims) {
+        // a record the trace did not write (its watchdog ran out)
+        atomicOr(sc.err, kErrHit);
+        done = true;
+    } else if (prim == kMiss) {
         radiance[3 * i] = __fmul_rn(fr, pd.sky[0]);
         radiance[3 * i + 1] = __fmul_rn(fg, pd.sky[1]);
         radiance[3 * i + 2] = __fmul_rn(fb, pd.sky[2]);

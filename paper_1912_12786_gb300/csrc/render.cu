@@ -287,7 +287,8 @@ __global__ void __launch_bounds__(256) k_render_backward_hits(
 // Shading of the saved hits, with the occlusion rays' any-hit records counted
 // on the way (pixel i's at i * spp .. i * spp + spp - 1; integers, so the count
 // does not depend on the traversal order); occ receives the occluded fraction
-// (0 for a miss).
+// (0 for a miss).  A primary record whose primitive is out of range gives the
+// background and is flagged (kErrHit).
 __global__ void __launch_bounds__(256) k_ao_shade(DevScene sc, ShadeDev sh,
                                                   const float4* __restrict__ hits,
                                                   const float4* __restrict__ ao_hits,
@@ -300,7 +301,9 @@ __global__ void __launch_bounds__(256) k_ao_shade(DevScene sc, ShadeDev sh,
     const uint32_t prim = __float_as_uint(h.w);
     float c[3] = {sh.bg[0], sh.bg[1], sh.bg[2]};
     float o = 0.0f;
-    if (prim != kMiss) {
+    if (prim != kMiss && prim >= sc.nprims) {
+        atomicOr(sc.err, kErrHit);
+    } else if (prim != kMiss) {
         uint32_t occluded = 0;
         for (uint32_t k = 0; k < spp; ++k)
             occluded += __float_as_uint(VSR_LDG(ao_hits + i * spp + k).w) != kMiss;

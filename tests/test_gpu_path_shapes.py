@@ -47,3 +47,19 @@ def test_watchdog_of_a_caller_who_asked_for_no_persistent_launch(V, small):
     got = _paths(V, small, n, V.trace_params(watchdog_iterations=3, watchdog_ms=1))
     assert V.vsr_get_device_error(small[1]) == 0
     assert torch.equal(got[1], want[1]) and torch.equal(got[0], want[0])
+
+
+def test_paths_that_the_watchdog_left_untraced(V, small):
+    """A persistent launch that stops at its budget leaves records that nothing
+    wrote: the shading takes no primitive id from them unchecked, the call
+    reports the timeout, and the next one is right."""
+    want = _paths(V, small, 200_001, V.trace_params())
+    for kw in (dict(lockstep=0), dict(lockstep=1, block_size=64)):
+        cut = V.trace_params(persistent=1, refill_threshold=16, watchdog_iterations=1, **kw)
+        rad, seg = _paths(V, small, 200_001, cut)
+        err = V.vsr_get_device_error(small[1])
+        assert err & V.DEVERR_TIMEOUT and err & ~(V.DEVERR_TIMEOUT | V.DEVERR_HIT) == 0, hex(err)
+        assert int(seg.min()) >= 1 and int(seg.max()) <= 3
+    got = _paths(V, small, 200_001, V.trace_params())
+    assert V.vsr_get_device_error(small[1]) == 0
+    assert torch.equal(got[1], want[1]) and torch.equal(got[0], want[0])
