@@ -549,8 +549,10 @@ vsr_status vsr_trace_persistent_noalloc(vsr_scene* scene, const vsr_ray* rays, u
  * ray in flight and to scene 0).
  *
  * vsr_batch_launch: the first call synchronises `stream`, tunes if needed,
- * runs the batch once and captures the launch (counter reset + kernel) in a
- * CUDA graph; every call then replays the graph on `stream`.  The recorded
+ * runs the batch once and captures the launch (a small kernel that resets the
+ * counter and reads the scenes' root boxes, and the trace) in a CUDA graph;
+ * every call then replays the graph on `stream`, so that it traces the scenes as
+ * vsr_scene_update has left them.  The recorded
  * pointers must stay valid for the batch's lifetime; the first launch writes
  * the hits more than once.  Errors: VSR_ERR_ARG, VSR_ERR_STATE (a scene
  * without BVH), VSR_ERR_OOM, VSR_ERR_CUDA.  nbatch is 1..65536.
@@ -696,7 +698,9 @@ vsr_status vsr_render_ao_backward(vsr_scene* scene, const vsr_hit* hits, const f
  * device data (same sizes as at creation; NULL leaves them unchanged).  After
  * a vertex update the triangle layout is rebuilt and the BVH boxes are refit
  * bottom-up (topology kept), so traces stay exact; traversal order and
- * bvh_costs counts then follow the refit boxes.  Synchronous.
+ * bvh_costs counts then follow the refit boxes.  Synchronous.  Batches follow
+ * updates; other launches that a caller recorded in a CUDA graph keep the root
+ * box of their recording and have to be recorded again.
  */
 vsr_status vsr_scene_update(vsr_scene* scene, const float* verts, uint32_t tex_index,
                             const void* texels, vsr_stream stream);

@@ -1862,6 +1862,7 @@ extern "C" vsr_status vsr_batch_create(vsr_scene* const* scenes, const vsr_ray* 
                                                   std::to_string(k) + ")");
         }
         items[k].sc = s->dev;
+        items[k].live = s->d_user;
         items[k].rays = reinterpret_cast<const float4*>(rays[k]);
         items[k].hits = reinterpret_cast<float4*>(hits[k]);
         offsets[k + 1] = offsets[k] + n[k];

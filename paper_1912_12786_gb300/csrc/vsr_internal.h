@@ -240,9 +240,12 @@ cudaError_t launch_render_backward_hits(const DevScene& sc, const ShadeDev& sh,
 // Source line of the first misaligned load a render kernel skipped (0 if
 // none), cleared after reading.
 cudaError_t render_align_error(unsigned* line);
-// One scene of a batched launch: its descriptor and its ray and hit arrays.
+// One scene of a batched launch: its descriptor (a copy, the items side by side
+// in L1), the scene's own in device memory, whose root box each refit renews,
+// and the ray and hit arrays.
 struct BatchItem {
     DevScene sc;
+    const DevScene* live;
     const float4* rays;
     float4* hits;
 };
@@ -259,7 +262,7 @@ struct SortTile {
 constexpr uint32_t kSortTileRays = 4096;
 
 struct BatchLaunch {
-    const BatchItem* items;             // device [nbatch]
+    BatchItem* items;                   // device [nbatch]
     const unsigned long long* offsets;  // device [nbatch + 1] ray prefix offsets
     uint32_t nbatch;
     IsectParams ip;
