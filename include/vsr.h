@@ -555,7 +555,8 @@ vsr_status vsr_trace_persistent_noalloc(vsr_scene* scene, const vsr_ray* rays, u
  * vsr_scene_update has left them.  The recorded
  * pointers must stay valid for the batch's lifetime; the first launch writes
  * the hits more than once.  Errors: VSR_ERR_ARG, VSR_ERR_STATE (a scene
- * without BVH), VSR_ERR_OOM, VSR_ERR_CUDA.  nbatch is 1..65536.
+ * without BVH; at a launch, a scene that was destroyed or given another BVH
+ * since the batch was created), VSR_ERR_OOM, VSR_ERR_CUDA.  nbatch is 1..65536.
  */
 typedef struct vsr_batch vsr_batch;
 
@@ -571,7 +572,7 @@ vsr_status vsr_batch_destroy(vsr_batch* batch);
 
 /*
  * One-call form: the library keeps the last 8 batches keyed by every
- * argument and launches the matching one, creating (and tuning) it on first
+ * argument (a scene by the BVH it holds, not by its address) and launches the matching one, creating (and tuning) it on first
  * use; make that first call outside any stream capture.
  */
 vsr_status vsr_trace_batch(vsr_scene* const* scenes, const vsr_ray* const* rays,

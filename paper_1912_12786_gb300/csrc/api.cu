@@ -3,12 +3,14 @@
 // arguments on the host before anything is launched, so an invalid call
 // returns an error instead of reaching a kernel.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstdint>
 #include <cstring>
 #include <limits>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -17,6 +19,14 @@
 #include "vsr_internal.h"
 
 using namespace vsr;
+
+// One loaded BVH, known to the batches made over it, which hold its device
+// memory's addresses: its id is never used again, and `alive` ends with it.
+struct LoadedBvh {
+    uint64_t id;
+    std::atomic<bool> alive{true};
+    explicit LoadedBvh(uint64_t i) : id(i) {}
+};
 
 struct vsr_scene {
     int device = 0;
@@ -32,6 +42,7 @@ struct vsr_scene {
     uint32_t num_nodes = 0, max_depth = 0;
     uint64_t records_up_to = 0;  // records_limit of the tree
     bool has_bvh = false;
+    std::shared_ptr<LoadedBvh> bvh;  // while has_bvh
     bool pooled = false;  // counted by the scratch pool
     DevScene dev{};
     DevScene* d_user = nullptr;
@@ -285,7 +296,15 @@ __global__ void k_ao_rays(const float* __restrict__ verts, const uint32_t* __res
     }
 }
 
+std::atomic<uint64_t> g_bvhs_loaded{0};
+std::atomic<uint64_t> g_bvhs_freed{0};
+
 void free_bvh(vsr_scene* s) {
+    if (s->bvh) {
+        s->bvh->alive = false;
+        s->bvh.reset();
+        ++g_bvhs_freed;
+    }
     dfree(s->d_nodes);
     dfree(s->d_wide);
     dfree(s->d_tris);
@@ -850,6 +869,7 @@ vsr_status vsr_bvh_load(vsr_scene* s, const void* blob, size_t bytes) {
         free_bvh(s);
         return cuda_fail(e, "scene descriptor upload");
     }
+    s->bvh = std::make_shared<LoadedBvh>(++g_bvhs_loaded);
     s->has_bvh = true;
     return VSR_OK;
 }
@@ -1578,6 +1598,8 @@ struct vsr_batch {
     IsectParams ip{};
     uint32_t stack_max = 1;
     bool records = true;  // every scene has two-level node records
+    std::vector<std::shared_ptr<LoadedBvh>> bvhs;  // the scenes', as recorded
+    uint64_t freed = 0;  // g_bvhs_freed when they were last seen alive
     BatchItem* d_items = nullptr;
     unsigned long long* d_offsets = nullptr;
     unsigned long long* d_work = nullptr;
@@ -1881,7 +1903,12 @@ extern "C" vsr_status vsr_batch_create(vsr_scene* const* scenes, const vsr_ray* 
     b->query = query;
     b->ip = isect_params(is);
     b->stack_max = stack_max;
-    for (const BatchItem& it : items) b->records = b->records && it.sc.wide;
+    b->freed = g_bvhs_freed;
+    b->bvhs.reserve(nbatch);
+    for (uint32_t k = 0; k < nbatch; ++k) {
+        b->records = b->records && items[k].sc.wide;
+        b->bvhs.push_back(scenes[k]->bvh);
+    }
     b->shape = shape;
     b->params = prm;
     b->tuned = params != nullptr || tune_lookup(shape, &b->params);
@@ -1905,6 +1932,14 @@ extern "C" vsr_status vsr_batch_create(vsr_scene* const* scenes, const vsr_ray* 
 extern "C" vsr_status vsr_batch_launch(vsr_batch* b, vsr_stream stream) {
     g_err.clear();
     if (!b) return fail(VSR_ERR_ARG, "batch is null");
+    if (const uint64_t freed = g_bvhs_freed; freed != b->freed) {
+        for (uint32_t k = 0; k < b->nbatch; ++k)
+            if (!b->bvhs[k]->alive)
+                return fail(VSR_ERR_STATE, "scene " + std::to_string(k) +
+                                               " was destroyed or given another BVH after the "
+                                               "batch was created");
+        b->freed = freed;
+    }
     DeviceGuard g(b->device);
     cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
     if (!b->exec) {
@@ -1974,7 +2009,10 @@ extern "C" vsr_status vsr_trace_batch(vsr_scene* const* scenes, const vsr_ray* c
         return fail(VSR_ERR_ARG, "invalid batch arguments");
     uint64_t key = 1469598103934665603ull;
     for (uint32_t k = 0; k < nbatch; ++k) {
+        if (!scenes[k]) return fail(VSR_ERR_ARG, "scene " + std::to_string(k) + " is null");
+        // not its address alone, which another scene may have after it
         key = fnv_mix(key, reinterpret_cast<uintptr_t>(scenes[k]));
+        key = fnv_mix(key, scenes[k]->bvh ? scenes[k]->bvh->id : 0);
         key = fnv_mix(key, reinterpret_cast<uintptr_t>(rays[k]));
         key = fnv_mix(key, reinterpret_cast<uintptr_t>(hits[k]));
         key = fnv_mix(key, n[k]);
