@@ -186,8 +186,14 @@ typedef struct vsr_trace_params {
                                   limit.  Running out acts as above. */
     uint32_t reg_cap_blocks;   /* register budget of vsr_trace's kernels, for
                                   measurement: 0 = each kernel's own (static:
-                                  none; dynamic: 3 blocks for closest hit, 4
-                                  for any hit); 1 = none; 3 or 4 = compiled to
+                                  none, but 5 blocks for the octant kernels'
+                                  any-hit alpha masks, 4.5 for their others
+                                  and 4 for the record kernels, which the
+                                  library may choose; dynamic: 3 blocks for
+                                  closest hit, 4 for any hit); 1 = none (with
+                                  static dispatch, octant 0 and one ray per
+                                  thread with per-lane loops, the generic
+                                  kernel, on every tree); 3 or 4 = compiled to
                                   fit that many 256-thread blocks per SM
                                   (static: one ray per thread with per-lane
                                   loops, stack_regs 0, intersectors default,

@@ -34,7 +34,9 @@ cudaError_t launch_static(const LaunchArgs& a, int kind, bool stats) {
     // 1,038, alpha mask 1,396 / 1,398; camera rays in rows gain 4 to 18%).  Any hit
     // in buffer order keeps the generic kernel, where rays that point anywhere are
     // 1 to 3% faster (default 927 / 955, alpha mask 1,322 / 1,344).
-    if (a.octant || (!a.persistent && !a.lockstep && a.stack_regs == 0 &&
+    // reg_cap 1 asks for a kernel without a register budget, which the octant
+    // kernels have: it gets the generic one, unless octant is asked for too.
+    if (a.octant || (!a.persistent && !a.lockstep && a.stack_regs == 0 && a.reg_cap == 0 &&
                      (a.query == kClosest || a.map.width > 0 ||
                       spreads_rays(a.map, kSpreadWarps))))
         return launch_static_octant(a, kind);

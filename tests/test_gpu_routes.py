@@ -1,0 +1,55 @@
+"""Which kernel a launch is routed to.  Every route gives the same result, so
+the choices that a caller makes through the launch parameters show only here."""
+import numpy as np
+import pytest
+
+from kernel_names import kernels_of
+from paper_1912_12786_gb300.inputs import scenes
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def V():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1912_12786_gb300 import _build, vsr
+    _build.build()
+    return vsr
+
+
+def _quads(n_quads):
+    rng = np.random.default_rng(n_quads)
+    side = 0.08 * (2048 / n_quads) ** 0.5
+    v, i, uv = scenes._quads_to_tris(scenes.random_quads(rng, n_quads, 0, 1, 0.2 * side, side))
+    return scenes.Scene("quads", v, i, uv, np.zeros(len(i), np.uint32), [scenes.disc_alpha_u8()])
+
+
+@pytest.fixture(scope="module", params=[2048, 100_000], ids=["short", "long"])
+def made(V, request):
+    """A tree with short and one with long descents, on which open launches
+    walk the two-level records."""
+    sc = _quads(request.param)
+    s = V.scene_from_inputs(sc, sc.bvh())
+    rays = scenes.pinhole_rays((0.5, 0.5, -1.0), (0.5, 0.5, 0.5), (0, 1, 0), 60.0, 320, 200)
+    yield request.param > 10_000, s, torch.from_numpy(rays).cuda()
+    s.close()
+
+
+def _trace(V, made, query, **kw):
+    _, s, d = made
+    hits = torch.empty(d.shape[0], 4, device="cuda")
+    return kernels_of(lambda st: V.vsr_trace(s, d, V.intersector("alpha_tex"), query, hits, None,
+                                             V.trace_params(**kw), st))
+
+
+@pytest.mark.parametrize("width", [0, 320])
+@pytest.mark.parametrize("query", ["closest", "any"])
+def test_no_register_budget_is_the_generic_kernel(V, made, query, width):
+    assert _trace(V, made, query, image_width=width, reg_cap_blocks=1) == ["k_trace"]
+    assert _trace(V, made, query, image_width=width, octant=1) == ["k_trace_oct"]
+    assert _trace(V, made, query, image_width=width, octant=1, reg_cap_blocks=1) == \
+        ["k_trace_oct"]
+    assert _trace(V, made, query, image_width=width) != ["k_trace"] or \
+        (query, width) == ("any", 0)
