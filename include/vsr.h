@@ -32,6 +32,10 @@
  *     allocations: a buffer carved from a larger allocation, as caching
  *     allocators do, is only checked against the enclosing allocation);
  *   - work is enqueued on the given stream and is asynchronous unless stated;
+ *   - scratch "from the stream-ordered allocator" comes from a memory pool that
+ *     the library has per CUDA context while scenes live there, allocated and
+ *     freed on the caller's stream; the pool keeps up to 512 MiB between calls
+ *     and gives it back when the last scene is destroyed;
  *   - CUDA failures map to VSR_ERR_CUDA, allocation failures to VSR_ERR_OOM.
  *
  * Floating point: the triangle and box tests use FP32 with a fixed rounding

@@ -43,7 +43,7 @@ struct vsr_scene {
     uint64_t records_up_to = 0;  // records_limit of the tree
     bool has_bvh = false;
     std::shared_ptr<LoadedBvh> bvh;  // while has_bvh
-    bool pooled = false;  // counted by the scratch pool
+    unsigned long long pooled = 0;  // the scratch pool's note of it
     DevScene dev{};
     DevScene* d_user = nullptr;
     uint32_t* d_err = nullptr;  // [0] device error word; [1] refit box state
@@ -741,8 +741,7 @@ vsr_status vsr_scene_create_indexed(const float* verts, uint32_t nverts, const u
             return bail(cuda_fail(e, "texture upload"));
     }
     s->h_tex = td;
-    scratch_scene_created();
-    s->pooled = true;
+    s->pooled = scratch_scene_created();
     *out = s;
     return VSR_OK;
 }
@@ -770,7 +769,7 @@ vsr_status vsr_scene_destroy(vsr_scene* s) {
     dfree(s->d_texels);
     dfree(s->d_user);
     dfree(s->d_err);
-    if (s->pooled) scratch_scene_destroyed();
+    scratch_scene_destroyed(s->pooled);
     delete s;
     return VSR_OK;
 }

@@ -1,14 +1,15 @@
-// Scratch from a stream-ordered pool of the library's own, one per device.
+// Scratch from a stream-ordered pool of the library's own, one per context.
 //
 // The device's default pool gives its memory back to the system at every
 // synchronisation, so a program that waits for each frame pays for mapping the
 // scratch again on each call (a persistent trace's 8-byte counter: 200 us).
 // This pool keeps up to kKeepBytes across synchronisations.  It exists while
-// scenes do: the last scene's destruction on a device returns what it holds.
+// scenes do: the last scene's destruction in a context returns what it holds.
 // Allocation and freeing are ordered on the caller's stream, as with the
 // default pool, so calls on several streams and threads do not share memory
 // that is in use.
 #include <mutex>
+#include <vector>
 
 #include "vsr_internal.h"
 
@@ -17,31 +18,28 @@ namespace vsr {
 namespace {
 
 constexpr unsigned long long kKeepBytes = 512ull << 20;
-constexpr int kDevices = 64;
 
+// A context is on one device, and its id is not used again: the entry of one
+// that has ended, with scenes alive or not, is never looked at again.
 struct Pool {
-    cudaMemPool_t pool = nullptr;
-    unsigned long long ctx = 0;  // id of the context it belongs to
-    unsigned long long scenes = 0;
+    unsigned long long ctx;
+    cudaMemPool_t pool;  // null: none could be made, the default pool serves
+    unsigned long long scenes;
 };
 std::mutex g_mutex;
-Pool g_pools[kDevices];
+std::vector<Pool> g_pools;
 
-// The current device's pool, made on first use; null where there is none (the
-// default pool serves then).  `make`: not on a stream under capture.
-cudaMemPool_t current_pool(int* device, bool make) {
-    unsigned long long ctx = 0;
-    if (cudaGetDevice(device) != cudaSuccess || *device < 0 || *device >= kDevices ||
-        !current_context_id(&ctx))
-        return nullptr;
-    Pool& p = g_pools[*device];
-    if (p.pool && p.ctx == ctx) return p.pool;
-    p.pool = nullptr;  // its context is gone, and it with it
-    if (!make) return nullptr;
+Pool* pool_of(unsigned long long ctx) {
+    for (Pool& p : g_pools)
+        if (p.ctx == ctx) return &p;
+    return nullptr;
+}
+
+cudaMemPool_t make_pool() {
     cudaMemPoolProps props{};
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = *device;
+    if (cudaGetDevice(&props.location.id) != cudaSuccess) return nullptr;
     cudaMemPool_t made = nullptr;
     unsigned long long keep = kKeepBytes;
     if (cudaMemPoolCreate(&made, &props) != cudaSuccess) {
@@ -53,37 +51,42 @@ cudaMemPool_t current_pool(int* device, bool make) {
         cudaMemPoolDestroy(made);
         return nullptr;
     }
-    p.pool = made;
-    p.ctx = ctx;
     return made;
 }
 
 }  // namespace
 
 cudaError_t scratch_alloc(void** ptr, size_t bytes, cudaStream_t stream) {
-    cudaMemPool_t pool;
-    {
+    cudaMemPool_t pool = nullptr;
+    unsigned long long ctx = 0;
+    if (current_context_id(&ctx)) {
         std::lock_guard<std::mutex> lock(g_mutex);
-        int device = 0;
-        pool = current_pool(&device, false);
+        if (const Pool* p = pool_of(ctx)) pool = p->pool;
     }
     return pool ? cudaMallocFromPoolAsync(ptr, bytes, pool, stream)
                 : cudaMallocAsync(ptr, bytes, stream);
 }
 
-void scratch_scene_created() {
+unsigned long long scratch_scene_created() {
+    unsigned long long ctx = 0;
+    if (!current_context_id(&ctx)) return 0;
     std::lock_guard<std::mutex> lock(g_mutex);
-    int device = 0;
-    current_pool(&device, true);
-    if (device >= 0 && device < kDevices) ++g_pools[device].scenes;
+    Pool* p = pool_of(ctx);
+    if (!p) {
+        g_pools.push_back(Pool{ctx, nullptr, 0});
+        p = &g_pools.back();
+    }
+    if (!p->pool) p->pool = make_pool();
+    ++p->scenes;
+    return ctx + 1;
 }
 
-void scratch_scene_destroyed() {
+void scratch_scene_destroyed(unsigned long long noted) {
+    unsigned long long ctx = 0;
+    if (!noted || !current_context_id(&ctx) || ctx + 1 != noted) return;
     std::lock_guard<std::mutex> lock(g_mutex);
-    int device = 0;
-    cudaMemPool_t pool = current_pool(&device, false);
-    if (device < 0 || device >= kDevices || g_pools[device].scenes == 0) return;
-    if (--g_pools[device].scenes == 0 && pool) cudaMemPoolTrimTo(pool, 0);
+    Pool* p = pool_of(ctx);
+    if (p && p->scenes && --p->scenes == 0 && p->pool) cudaMemPoolTrimTo(p->pool, 0);
 }
 
 }  // namespace vsr

@@ -122,10 +122,11 @@ inline bool spreads_rays(RayMap map, unsigned warps_per_sm) {
 }
 
 // Stream-ordered scratch (scratch.cu), freed with cudaFreeAsync.  The pool lives
-// while scenes do; both notes are for the current device.
+// while scenes do: a scene's creation notes the current context (0: not counted),
+// and its destruction hands the note back.
 cudaError_t scratch_alloc(void** ptr, size_t bytes, cudaStream_t stream);
-void scratch_scene_created();
-void scratch_scene_destroyed();
+unsigned long long scratch_scene_created();
+void scratch_scene_destroyed(unsigned long long noted);
 // Unique id of the calling thread's current CUDA context (ids are never reused
 // within a process).
 bool current_context_id(unsigned long long* id);
