@@ -14,9 +14,12 @@ Also reported: a per-intersector breakdown (default, alpha texture,
 procedural alpha, counting; static and dynamic dispatch), the roofline of the
 dominant kernel from exact algorithmic bytes, an end-to-end number with host
 buffers, clocks sampled during the timed region and the CPU oracle timed on a
-bounded sample of the same workload.
+bounded sample of the same workload.  One short JSON line on stdout holds the
+headline; everything else goes to stderr as one JSON line, and with --details
+to a file.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
+                  [--details FILE]
 """
 from __future__ import annotations
 
@@ -378,6 +381,37 @@ def launch_config(p) -> str:
     return s
 
 
+# the most that a launcher which keeps only the end of the output will hold
+LINE_LIMIT = 1480
+
+
+def headline(out: dict) -> str:
+    """The stdout line: the headline's keys of a full result, below LINE_LIMIT
+    characters (the full result takes 16,000)."""
+    def pick(d, *keys):
+        return {k: d[k] for k in keys if k in d} if d else d
+
+    c = out["config"]
+    short = {k: out[k] for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup",
+                                 "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+                                 "dtype", "data")}
+    short["config"] = pick(c, "workload", "rays_per_step", "launch", "primary", "shadow", "l2",
+                           "parallelism")
+    short["roofline"] = pick(out.get("roofline"), "bound", "achieved", "peak", "unit", "frac",
+                             "kernel")
+    short["gpu_launches"] = out["gpu_launches"]
+    short["clocks"] = pick(out.get("clocks"), "sm_mhz", "sm_max_mhz", "reasons")
+    short["e2e"] = pick(out["e2e"], "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step")
+    if out.get("fwd_bwd"):
+        short["fwd_bwd"] = pick(out["fwd_bwd"], "value", "unit")
+    if out.get("cpu_baseline"):
+        short["cpu_baseline"] = pick(out["cpu_baseline"], "value", "unit", "cores", "kind")
+    line = json.dumps(short)
+    if len(line) > LINE_LIMIT:
+        raise ValueError(f"the result line has {len(line)} characters")
+    return line
+
+
 def profiled_levels(kernel: str, config: str):
     """Per-launch bytes at each memory level from the committed ncu summary
     of `kernel` -- L1 (l1tex__t_sectors x 32), L2 (lts__t_sectors x 32) and
@@ -722,13 +756,11 @@ def run_ours(args):
            "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
            "config": {"workload": WORKLOAD, "rays_per_step": rays_per_step,
                       "triangles": sc.ntri,
-                      "launch": ("vsr_trace with params NULL: the configuration "
-                                 "vsr_trace_tune chose on the frame (untimed, before the steps)"
+                      "launch": ("params NULL, tuned on the frame before the steps"
                                  if args.launch == "tuned" else
-                                 "vsr_trace with the octant configuration passed explicitly "
-                                 "(--launch octant; nothing tuned)"),
-                      "tuned_primary": V.params_dict(tuned_p),
-                      "tuned_shadow": V.params_dict(tuned_s),
+                                 "octant configuration passed (--launch octant)"),
+                      "primary": launch_config(tuned_p),
+                      "shadow": launch_config(tuned_s),
                       "ray_order": "row-major frame; each warp traces a 4x8 pixel tile",
                       "l2": "flushed between steps (256 MiB write)",
                       "parallelism": f"replicas x{world} (each rank traces its own frame)"},
@@ -878,7 +910,12 @@ def run_ours(args):
                                                        f"({nsel1} + {nsel1} rays) x {reps1} "
                                                        f"repeats, {el1:.1f} s"}
     if rank == 0:
-        print(json.dumps(out), flush=True)
+        full = json.dumps(out)
+        print(full, file=sys.stderr, flush=True)
+        if args.details:
+            with open(args.details, "w") as f:
+                f.write(full + "\n")
+        print(headline(out), flush=True)
     s.close()
     if world > 1:
         import torch.distributed as dist
@@ -1520,6 +1557,8 @@ def main():
     ap.add_argument("--impl", choices=["ours", "reference"], default="ours")
     ap.add_argument("--ref-stride", type=int, default=1)
     ap.add_argument("--no-breakdown", action="store_true")
+    ap.add_argument("--details", metavar="FILE",
+                    help="also write the full result (stderr's JSON line) there")
     ap.add_argument("--no-cpu", action="store_true")
     ap.add_argument("--leg", choices=["all", "large", "batch", "fwd_bwd", "trace", "ao",
                                       "ao_bwd", "batch_profile"],
