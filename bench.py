@@ -65,7 +65,9 @@ E2E_TRACE_STREAMS = 4  # streams the bands' traces go to, round robin
 def default_params(V, image_width=FRAME_W):
     """Launch configuration of the per-intersector comparisons (and the
     full-size test): one ray per thread, warps on 4x8 pixel tiles of the
-    row-major frame, the generic box test (either dispatch)."""
+    row-major frame.  The static kernels then specialise the box test to a
+    warp's direction octant where its rays share one; the callback kernels use
+    the generic test.  Like for like: the legs with reg_cap_blocks."""
     return V.trace_params(block_size=128, persistent=0, refill_threshold=16,
                           image_width=image_width)
 
@@ -965,9 +967,10 @@ def breakdown(V, s, d_rays, rays_s, n, flush, stream, torch, reps=5):
             res[f"{q}/{kind}/overhead_vs_default"] = round(base / res[f"{q}/{kind}/static"] - 1, 4)
             res[f"{q}/{kind}/dynamic_vs_static"] = round(
                 res[f"{q}/{kind}/static"] / res[f"{q}/{kind}/dynamic"], 4)
-    # static vs dynamic injection at equal register budgets: both kernels
-    # compiled with __launch_bounds__(256, b) for b = 3 and 4, and both
-    # without a budget (b = 1); shared-memory stack, same tiles
+    # static vs dynamic injection, and nothing else: both kernels with the
+    # generic box test and per-lane loops, compiled with
+    # __launch_bounds__(256, b) for b = 3 and 4, and both without a budget
+    # (b = 1); shared-memory stack, same tiles
     for q, rr in (("closest", d_rays), ("any", rays_s)):
         for kind in ("default", "alpha_tex", "proc_alpha", "count"):
             c = cnt if kind == "count" else None
@@ -998,7 +1001,9 @@ def breakdown(V, s, d_rays, rays_s, n, flush, stream, torch, reps=5):
     alpha = V.intersector("alpha_tex")
     for block in (64, 128, 256):
         for k in (0, 1, 2, 4, 8):
-            p = V.trace_params(block_size=block, image_width=FRAME_W, stack_regs=k)
+            # reg_cap_blocks 1 keeps the generic kernel for K = 0 as well
+            p = V.trace_params(block_size=block, image_width=FRAME_W, stack_regs=k,
+                               reg_cap_blocks=1)
             for q, rr in (("closest", d_rays), ("any", rays_s)):
                 ms = []
                 for r in range(reps + 2):
@@ -1098,7 +1103,7 @@ def path_bench(V, s, sc, d_rays, n, flush, stream, torch, steps, bounces=3):
             "segments": segments, "Msegments_s": round(segments / (t / 1e3) / 1e6, 1),
             "lockstep_persistent_ms_per_frame": round(tl, 4),
             "lockstep_persistent_Mpaths_s": round(n / (tl / 1e3) / 1e6, 1),
-            "gpu_launches_per_frame": 1 + 2 * (bounces + 1) + 3 * bounces}
+            "gpu_launches_per_frame": 2 * (bounces + 1)}
 
 
 def instanced_bench(V, torch, dev, flush, stream, steps):
