@@ -54,5 +54,6 @@ def _name(cu, node):
     else:
         _check(cu.cuKernelGetName(ctypes.byref(text), ctypes.c_void_p(words[7])), "kernel name")
     mangled = text.value.decode()
-    m = re.search(r"(\d+)(k_\w+)", mangled)
-    return m.group(2)[:int(m.group(1))] if m else mangled
+    # the name in lower case, up to the template's or the signature's letter
+    m = re.search(r"\dk_[a-z0-9_]+", mangled)
+    return m.group(0)[1:] if m else mangled
