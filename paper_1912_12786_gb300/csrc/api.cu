@@ -598,7 +598,7 @@ vsr_status tune_trace(vsr_scene* s, const LaunchArgs& base, const vsr_intersecto
             for (uint32_t k : {0u, 1u, 2u, 4u, 8u})
                 if ((!dynamic || k == 0) && !(b == 128u && k == 0u && ls == 0u))
                     consider(vsr_trace_params{b, 0u, 16u, 0u, image_width, k, 0u, 0u, 0u, 0u, ls});
-    if (!dynamic && query == kAny && image_width == 0)
+    if (!dynamic && image_width == 0 && (query == kAny || is->kind == VSR_ISECT_CLIP))
         // elsewhere the octant-dispatching kernel runs with octant 0 too
         for (uint32_t b : {64u, 128u, 256u}) {
             vsr_trace_params c{b, 0u, 16u, 0u, image_width, 0u, 0u, 0u, 0u, 0u, 0u};

@@ -14,6 +14,8 @@
 // Which launches of that shape run these kernels without asking for it (octant
 // 1): launch_static.  Camera rays gain (forest frame 524 -> 475 us, heat map of
 // 1283 x 719 154 -> 133 us), and the vote costs mixed warps nothing that shows.
+#include <type_traits>
+
 #include "trace_static.cuh"
 
 namespace vsr {
@@ -27,11 +29,16 @@ namespace {
 // rays, us without / with: closest default 1,056 / 985, procedural 1,466 / 1,399,
 // count 1,043 / 998, any count 1,004 / 945; 2,073,600 camera rays in rows on the
 // forest: default 378 / 371, procedural 602 / 586, any count 140 / 134.  The masks'
-// any hit at 36 warps instead of 40: 1,342 / 1,397.
+// any hit at 36 warps instead of 40: 1,342 / 1,397.  The clip box's closest hit
+// spills 20 bytes at 36 warps and gets 32 (63 registers): 518,400 camera rays on
+// tiles, forest 144 (generic kernel) / 132 us, 100,000 quads 205 / 193; at 36 warps
+// 4,000 quads took 81 / 89, now 83 / 84.
 template <int Q, class H>
 struct OctBudget {
     static constexpr bool kMask = Q == kAny && H::kTexcoords;
-    static constexpr int kThreads = kMask ? 256 : 384, kBlocks = kMask ? 5 : 3;
+    static constexpr bool kClip = Q == kClosest && std::is_same<H, IsectClip>::value;
+    static constexpr int kThreads = kMask || kClip ? 256 : 384;
+    static constexpr int kBlocks = kMask ? 5 : kClip ? 4 : 3;
 };
 
 template <int Q, class H>

@@ -33,11 +33,13 @@ cudaError_t launch_static(const LaunchArgs& a, int kind, bool stats) {
     // warps are no slower in it: 1,000,003 diffuse rays, default 985 us against
     // 1,038, alpha mask 1,396 / 1,398; camera rays in rows gain 4 to 18%).  Any hit
     // in buffer order keeps the generic kernel, where rays that point anywhere are
-    // 1 to 3% faster (default 927 / 955, alpha mask 1,322 / 1,344).
+    // 1 to 3% faster (default 927 / 955, alpha mask 1,322 / 1,344), and so does the
+    // clip box's closest hit there (518,400 diffuse rays, 100,000 quads 588 / 617 us,
+    // 4,000 quads 310 / 322; the forest's 1,440,000 3,354 / 3,477).
     // reg_cap 1 asks for a kernel without a register budget, which the octant
     // kernels have: it gets the generic one, unless octant is asked for too.
     if (a.octant || (!a.persistent && !a.lockstep && a.stack_regs == 0 && a.reg_cap == 0 &&
-                     (a.query == kClosest || a.map.width > 0 ||
+                     ((a.query == kClosest && kind != 5) || a.map.width > 0 ||
                       spreads_rays(a.map, kSpreadWarps))))
         return launch_static_octant(a, kind);
     switch (a.stack_regs) {

@@ -53,3 +53,25 @@ def test_no_register_budget_is_the_generic_kernel(V, made, query, width):
         ["k_trace_oct"]
     assert _trace(V, made, query, image_width=width) != ["k_trace"] or \
         (query, width) == ("any", 0)
+
+
+def test_clip_box_closest_hit(V):
+    """The generic kernel in buffer order, where its rays are faster, the octant
+    kernel on tiles and for few rays."""
+    sc, rays = scenes.small_quads(res=320)
+    s = V.scene_from_inputs(sc, sc.bvh())
+    d = torch.from_numpy(rays).cuda()
+    hits = torch.empty(len(rays), 4, device="cuda")
+    isect = V.intersector("clip", clip_lo=(0.2, 0.1, 0.0), clip_hi=(0.8, 0.7, 0.9))
+    out = []
+    for n, width, kernel in ((len(rays), 0, "k_trace"), (len(rays), 320, "k_trace_oct"),
+                             (2000, 0, "k_trace_oct")):
+        p = V.trace_params(image_width=width)
+        names = kernels_of(lambda st: V.vsr_trace(s, d[:n], isect, "closest", hits[:n], None, p,
+                                                  st))
+        assert names == [kernel]
+        V.vsr_trace(s, d[:n], isect, "closest", hits[:n], None, p)
+        torch.cuda.synchronize()
+        out.append(hits[:n].clone().view(torch.int32))
+    assert torch.equal(out[0], out[1]) and torch.equal(out[0][:2000], out[2])
+    s.close()
