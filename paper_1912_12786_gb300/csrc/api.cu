@@ -346,6 +346,18 @@ uint64_t records_limit(const vsr_bvh_node* nodes, uint32_t num_nodes) {
     return visits >= 90.0 ? (uint64_t)std::min(32.0 * visits * visits, 1e15) : 0;
 }
 
+// Whether the records stand for the boxes as they are (write_wide_header, which
+// notes the same for the kernels).  Where they do not, each ray of a record kernel
+// walks the binary nodes by itself; the launches below take the binary kernels
+// instead.  500,000 diffuse rays on 200,000 triangles, vertices scaled by 1e12,
+// alpha texture, any hit, us record / binary kernels: open form 838 / 736,
+// persistent lock step 789 / 473, batch 818 / 499.
+bool records_hold(const DevScene& d) {
+    constexpr float kExtent = 0x1p35f;
+    return d.boxes_ordered && d.root_b.x - d.root_a.x <= kExtent &&
+           d.root_b.y - d.root_a.y <= kExtent && d.root_b.z - d.root_a.z <= kExtent;
+}
+
 vsr_status validate_isect(const vsr_intersector* is, int32_t query) {
     if (!is) return fail(VSR_ERR_ARG, "intersector is null");
     if (is->kind < VSR_ISECT_NONE || is->kind > VSR_ISECT_CLIP)
@@ -484,7 +496,8 @@ vsr_status prepare_launch(vsr_scene* s, const vsr_ray* rays, uint64_t n,
     a.query = query;
     a.work = nullptr;  // persistent launches take their own counter
     a.dyn_user = s->d_user;
-    a.records_up_to = s->records_up_to;
+    if (!records_hold(a.sc)) a.sc.wide = nullptr;
+    a.records_up_to = a.sc.wide ? s->records_up_to : 0;
     return VSR_OK;
 }
 
@@ -1596,7 +1609,7 @@ struct vsr_batch {
     int kind = 0, query = 0;
     IsectParams ip{};
     uint32_t stack_max = 1;
-    bool records = true;  // every scene has two-level node records
+    bool records = true;  // every scene has two-level node records, in use
     std::vector<std::shared_ptr<LoadedBvh>> bvhs;  // the scenes', as recorded
     uint64_t freed = 0;  // g_bvhs_freed when they were last seen alive
     BatchItem* d_items = nullptr;
@@ -1905,7 +1918,7 @@ extern "C" vsr_status vsr_batch_create(vsr_scene* const* scenes, const vsr_ray* 
     b->freed = g_bvhs_freed;
     b->bvhs.reserve(nbatch);
     for (uint32_t k = 0; k < nbatch; ++k) {
-        b->records = b->records && items[k].sc.wide;
+        b->records = b->records && items[k].sc.wide && records_hold(items[k].sc);
         b->bvhs.push_back(scenes[k]->bvh);
     }
     b->shape = shape;

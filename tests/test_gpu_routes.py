@@ -75,3 +75,23 @@ def test_clip_box_closest_hit(V):
         out.append(hits[:n].clone().view(torch.int32))
     assert torch.equal(out[0], out[1]) and torch.equal(out[0][:2000], out[2])
     s.close()
+
+
+def test_record_kernels_only_where_the_records_hold(V, made):
+    """After updates that leave boxes non-finite or the grid too coarse, lock
+    step takes the binary kernels, and the record kernels again after the next."""
+    long, s, d = made
+    sc = _quads(100_000 if long else 2048)
+    base = torch.from_numpy(sc.verts).cuda()
+    nan = base.clone()
+    nan[5] = float("nan")
+    bad = nan.clone()
+    bad[torch.from_numpy(sc.idx[:200].astype(np.int64).ravel()).cuda()] = float("nan")
+    shapes = (dict(lockstep=1), dict(lockstep=1, persistent=1), dict())
+    wide = ["k_trace_wide", "k_trace_wide_persistent", "k_trace_wide"]
+    binary = ["k_trace_ls", "k_trace_persistent", "k_trace_oct"]
+    for verts, holds in ((base, True), (bad, False), (base * 1e12, False), (nan, True),
+                         (base, True)):
+        V.vsr_scene_update(s, verts.contiguous())
+        got = [_trace(V, made, "closest", **kw)[-1] for kw in shapes]
+        assert got == (wide if holds and long else binary)
