@@ -28,6 +28,7 @@ import hashlib
 import json
 import math
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -90,13 +91,15 @@ TRACE_SOURCES = ("trace_static.cuh", "vsr_device.cuh", "trace_oct.cu", "wide.cuh
 
 
 def kernel_source_hash() -> str:
-    """Hash of the sources the static trace kernels compile from: profiled
-    counters are used only while it matches the committed summary's."""
+    """Hash of the sources the static trace kernels compile from, without their
+    comments: profiled counters are used only while it matches the committed
+    summary's."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1912_12786_gb300", "csrc")
     for f in TRACE_SOURCES:
-        with open(os.path.join(csrc, f), "rb") as fh:
-            h.update(f.encode() + fh.read())
+        with open(os.path.join(csrc, f), encoding="utf-8") as fh:
+            code = re.sub(r"//[^\n]*|/\*.*?\*/", " ", fh.read(), flags=re.S)
+        h.update(f.encode() + " ".join(code.split()).encode())
     return h.hexdigest()[:16]
 
 

@@ -373,8 +373,10 @@ vsr_status vsr_trace_tuned_params(vsr_scene* scene, const vsr_intersector* isect
  *   params    one ray per thread, or persistent warps (persistent 1, refill
  *             threshold, blocks per SM, watchdog as for vsr_trace) with
  *             per-lane loops or in lock step (lockstep 1 takes persistent
- *             1); image_width allowed; stack in shared memory (stack_regs
- *             ignored).  Results are identical in every configuration.
+ *             1; with persistent 0 the library runs static launches of eight
+ *             and more rays per warp in lock step); image_width allowed; stack
+ *             in shared memory (stack_regs ignored).  Results are identical in
+ *             every configuration.
  * Errors as vsr_trace.
  */
 vsr_status vsr_trace_multi(vsr_scene* scene, const vsr_ray* rays, uint64_t n,
@@ -402,9 +404,13 @@ vsr_status vsr_trace_multi(vsr_scene* scene, const vsr_ray* rays, uint64_t n,
  *   radiance  device float32 [n * 3], written
  *   segments  device uint32 [n] or NULL: closest-hit queries path i made
  *   params    every segment's launch; image_width maps the primary
- *             segments to pixel tiles; persistent launches and lock step
- *             apply to each segment depth (with neither, segments after a
- *             bounce may use them); ray_order 0
+ *             segments to pixel tiles; persistent launches, lock step,
+ *             stack_regs and reg_cap_blocks apply to each segment depth.  With
+ *             none of them, the library chooses the form of the static
+ *             segments after a bounce, octant 1 or not (lock step, from three
+ *             waves of threads on persistent, without the watchdog);
+ *             reg_cap_blocks 1 keeps per-lane loops, one ray per thread, on
+ *             every segment; ray_order 0
  * One closest-hit launch per segment depth plus one shading launch, on
  * `stream`.  The shading launch also lists the paths that go on (their order
  * may vary from run to run; results do not depend on it), and the next

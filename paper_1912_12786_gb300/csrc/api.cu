@@ -321,7 +321,8 @@ void free_bvh(vsr_scene* s) {
 // ray descends through many boxes per leaf, because lanes then reach their
 // leaves far apart even when neighbouring rays agree; the surface areas of the
 // boxes tell, relative to the root's the expected visits of a ray that crosses
-// the scene: `inner` nodes, and inner per leaf.  Closest hit, alpha texture, us
+// the scene: `inner` nodes, and inner per leaf.  They are those of the tree as
+// loaded; a refit does not change the limit.  Closest hit, alpha texture, us
 // per-lane / lock step, camera rays 480 x 270, 960 x 540 and 1920 x 1080 and
 // 1,000,000 diffuse rays:
 //   random quads, 2,000,000 (inner 291, 36 per leaf)

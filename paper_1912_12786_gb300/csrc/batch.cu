@@ -15,7 +15,7 @@
 // order instead: slot k names the ray perm[k], and scene s still owns slots
 // [offsets[s], offsets[s+1]) because the sort key is scene-major.  Per-ray
 // results are identical to a per-scene vsr_trace: the traversal code is the
-// same (traverse_start / traverse_step).
+// same (traverse_step, warp_step, or wide_step over the records).
 #include "wide.cuh"
 
 namespace vsr {
@@ -227,6 +227,13 @@ cudaError_t batch_depth(const BatchLaunch& b, cudaStream_t stream, uint32_t* gri
     }
 }
 
+// Lock step walks the records if every scene has them, whatever its tree, and not
+// only where records_limit sends single launches: one kernel serves all scenes of a
+// batch, long trees and short.  That gains on random quads and costs on trees with
+// short descents, where the binary walk is there with stack_regs 2 and the tuner finds
+// it.  Block 64, refill 24, alpha texture, closest / any hit, us records / binary
+// nodes: 4 x 100,000 quads 356/362, 331/357; 20 x 3,000 quads 210/203, 192/193;
+// forests 6 x 20,002 780/690, 304/302; 3 x 200,002 992/854, 372/353.
 template <int Q, class H>
 cudaError_t batch_regs(const BatchLaunch& b, cudaStream_t stream, uint32_t* grid) {
     if constexpr (H::kWide)

@@ -240,6 +240,12 @@ cudaError_t multi_one(const LaunchArgs& a, const float* verts, const uint32_t* i
                           : multi_persistent<H, false>(a, verts, idx, nh);
     const size_t smem = ((size_t)a.sc.stack_depth + 2u * nh) * a.block * sizeof(uint32_t);
     RayMap map = a.map;
+    // The octant kernels' line, though the 63 or 64 registers here leave room for 32
+    // warps: a ray that keeps many hits gains more from fewer neighbours than a last
+    // wave costs.  Image tiles of 5,120, 20,480 and 81,920 rays, alpha texture, us
+    // with lines of 32 / 36 warps: 100,000 quads, 4 hits 124/98 181/148 226/197, 16
+    // hits 142/111 214/179 298/253; forest, 16 hits 359/263 541/492 687/644, but 1
+    // hit 93/89 128/130 130/148.
     const unsigned long long grid = (spread_rays(map, kSpreadWarps) + a.block - 1) / a.block;
     auto go = [&](auto k, auto... more) {
         if (smem > 48 * 1024) {

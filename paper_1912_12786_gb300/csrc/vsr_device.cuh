@@ -979,8 +979,10 @@ __device__ __forceinline__ bool watchdog_expired(const Watchdog& wd, uint32_t it
 // that divergent part.  The loop's exits (all lanes idle and the counter
 // passed the end, or the watchdog) are uniform decisions.  No lane waits on
 // another warp or block.  Each iteration claims at least one ray or advances
-// some lane's ray (bounded per ray by the traversal's own visit bound), so
-// the loop ends; the watchdog bounds it whatever happens.
+// some lane's ray, and a ray's visits are bounded: children follow their parent
+// (the loader's validator), so a descent ends, and leaves are counted (with
+// per-lane loops every node).  So the loop ends; the watchdog bounds the number
+// of its iterations whatever happens.
 template <bool LS, class Start, class Step, class Finish, class Fail>
 __device__ __forceinline__ void persistent_rays(const RayMap& map, unsigned long long* work,
                                                 uint32_t refill, const Watchdog& wd,

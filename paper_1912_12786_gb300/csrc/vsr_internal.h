@@ -94,7 +94,7 @@ inline int persistent_grid(const LaunchArgs& a, const void* kernel, size_t smem)
 // Random quads would take more warps, but neighbouring camera rays that agree
 // (the forest) lose once the warps no longer fit the chip at once: the line is
 // what stays resident, 36 warps of the octant kernels' 56 registers, 24 of the
-// kernels with 78 to 80.  In buffer order a warp's rays share less and every
+// kernels with 78 to 80 (multi-hit: trace_multi.cu).  In buffer order a warp's rays share less and every
 // further warp loads nodes of its own, from DRAM when the caches are cold (the
 // table above is warm), so there the line is 14 for all kernels: camera rays
 // through random pixels, forest of 200,002 triangles, L2 flushed, us with lines

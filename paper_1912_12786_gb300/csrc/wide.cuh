@@ -42,7 +42,7 @@
 //    popped, at the far limit of that moment, as there.  So every leaf
 //    traverse_body tests is tested here, in the same order;
 //  - a leaf more than those must not change the result: before a candidate is
-//    taken, its leaf's exact box is tested (wide_verdict).  If it is missed at
+//    taken, its leaf's exact box is tested (WideLane::test).  If it is missed at
 //    the ray's own limits, traverse_body never tests the leaf.  If it is hit at
 //    the far limit held when the leaf was reached here, traverse_body's limit
 //    was no smaller and it tests the leaf.  Between the two (the candidate lies
@@ -56,7 +56,10 @@
 // position).  The ray itself and the running result, needed at leaves only, are
 // in shared memory beside the stack (LaneStore), which takes the kernels from
 // 78-80 registers, 24 resident warps per SM, to 64 and 32 (closest hit 816 ->
-// 785 us below; at 48 registers they spill and lose a quarter).
+// 785 us below; at 48 registers they spill and lose a quarter).  At 64 the way
+// back to the binary nodes, inlined twice, still spills: 44 to 108 bytes in the
+// closest-hit kernels of one ray per thread, 46 in the persistent and 98 to 118 in
+// the batched ones, 8 to 40 with any hit.
 //
 // Measured against warp_step on the binary nodes (persistent, refill 24):
 // 1,000,003 diffuse rays on 200,000 triangles, alpha texture, closest 838 ->
